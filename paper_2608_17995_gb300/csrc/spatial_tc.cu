@@ -48,16 +48,21 @@
 //   warps 1, 18   MMA issuers, one per query tile: S = Q K^T with
 //                 tcgen05.mma kind::f16 (bf16 in, fp32 accumulate in tensor
 //                 memory), 128x128 per tile, two S buffers per Q tile (all 512
-//                 TMEM columns).  A barrier wait in the issuing thread costs
-//                 the tensor pipe a bubble; a second issuer fills it.
+//                 TMEM columns).  A barrier wait in the issuing warp costs
+//                 the tensor pipe a bubble; a second issuer fills it.  The
+//                 whole warp waits and one elected lane issues: the compiler
+//                 then keeps descriptors in uniform registers (4096 x 4608 x
+//                 24 heads 92.0 -> 89.2 us against a loop in lane 0 alone).
 //   warps 2-17    four softmax warpgroups: query tile t and column half c
 //                 (64 of the 128 keys of a tile) per warpgroup, so all 16
 //                 warps work on the same item while the MMA fills the other S
-//                 buffer; one TMEM lane (= one query row) per thread, 16
+//                 buffer; one TMEM lane (= one query row) per thread, 32
 //                 columns per tcgen05.ld, ex2 on the MUFU against the running
-//                 row maximum with packed f32x2 FMA/add.  The exact chunk
-//                 maximum is only computed when a chunk sum would leave
-//                 [0, 2^64) (first chunk, a larger logit, NaN).  The text keys
+//                 row maximum with packed f32x2 FMA/add.  The exact maximum of
+//                 the 32 is only computed when their sum would leave [0, 2^64)
+//                 (first keys, a larger logit, NaN).  32 at a time, load and
+//                 wait in one statement: 89.1 -> 84.0 us; 16 with the next 16
+//                 loading 89.1, 64 at a time 102.  The text keys
 //                 come first, so the text sum is a prefix of the row sum.  At
 //                 d = 128 a 128x128 tile costs the tensor pipe and the MUFU
 //                 (32 ex2 / clock / SM) the same 512 cycles; evaluating part
@@ -154,32 +159,29 @@ __device__ __forceinline__ void merge_stat(RowStat& a, float m2, float la2, floa
   a.m = m;
 }
 
-// One chunk of 16 keys that are all valid and all text (kText) or all image
-// keys: the common case, kept free of the masking and boundary logic (a
-// per-chunk branch on the key kind measured ~15% slower on the whole item).
+// 32 keys that are all valid and all text (kText) or all image keys: the
+// common case, kept free of the masking and boundary logic (a branch on the
+// key kind per 16 keys measured ~15% slower on the whole item).
 template <bool kText>
-__device__ __forceinline__ void process_chunk_full(const uint32_t (&r)[16], float c, RowStat& st) {
-  float v[16];
-#pragma unroll
-  for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(r[e]);
+__device__ __forceinline__ void process_cols_full(const uint32_t (&v)[32], float c, RowStat& st) {
   const float nm = -st.m;
   float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll
-  for (int e = 0; e < 16; e += 4) {
+  for (int e = 0; e < 32; e += 4) {
     float x0, x1, x2, x3;
-    ffma2(v[e], v[e + 1], c, nm, x0, x1);
-    ffma2(v[e + 2], v[e + 3], c, nm, x2, x3);
+    ffma2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), c, nm, x0, x1);
+    ffma2(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]), c, nm, x2, x3);
     fadd2(s0, s1, ex2(x0), ex2(x1));
     fadd2(s2, s3, ex2(x2), ex2(x3));
   }
   fadd2(s0, s1, s2, s3);
   float cs = s0 + s1;
   if (!(cs < 0x1p64f)) {
-    // first chunk of a row, a logit 64 log2-units above the running maximum,
-    // or a NaN: take the exact chunk maximum and rescale the running sums
-    float cm = v[0];
+    // first keys of a row, a logit 64 log2-units above the running maximum,
+    // or a NaN: take the exact maximum and rescale the running sums
+    float cm = __uint_as_float(v[0]);
 #pragma unroll
-    for (int e = 1; e < 16; ++e) cm = fmaxf(cm, v[e]);
+    for (int e = 1; e < 32; ++e) cm = fmaxf(cm, __uint_as_float(v[e]));
     const float mx = fmaxf(st.m, cm * c);
     const float corr = ex2(st.m - mx);
     st.la *= corr;
@@ -187,7 +189,7 @@ __device__ __forceinline__ void process_chunk_full(const uint32_t (&r)[16], floa
     st.m = mx;
     cs = 0.f;
 #pragma unroll
-    for (int e = 0; e < 16; ++e) cs += ex2(fmaf(v[e], c, -mx));
+    for (int e = 0; e < 32; ++e) cs += ex2(fmaf(__uint_as_float(v[e]), c, -mx));
   }
   st.la += cs;
   if (kText) st.lt += cs;
@@ -291,7 +293,7 @@ enum ItemKind { kItemImage = 0, kItemText = 1, kItemGeneral = 2, kItemMasked = 3
 
 // A chunk whose text keys are given by a mask (bit e = key col0 + e is a text
 // key), possibly with invalid keys beyond Nk: the mixed case of a caller's
-// key mask.  Same lazy running maximum as process_chunk_full; the text sum
+// key mask.  Same lazy running maximum as process_cols_full; the text sum
 // takes the exponentials of the masked keys.
 __device__ __forceinline__ void process_chunk_masked(const uint32_t (&r)[16], int col0, int Nk,
                                                      uint32_t m16, float c, RowStat& st) {
@@ -350,33 +352,33 @@ template <int kKind>
 __device__ __forceinline__ void softmax_item(uint32_t tb, int c0, int Nk, int L, float c,
                                              RowStat& st, uint64_t* s_empty, int lane,
                                              uint32_t w0 = 0u, uint32_t w1 = 0u) {
-  uint32_t ra[16], rb[16];
-  const int nch = (kKind >= kItemGeneral) ? max(0, min(4, (Nk - c0 + 15) >> 4)) : 4;
-  auto chunk = [&](const uint32_t(&r)[16], int k) {
-    if (kKind == kItemGeneral) {
-      if (k < nch) process_chunk(r, c0 + 16 * k, Nk, L, c, st);
-    } else if (kKind == kItemMasked) {
-      const uint32_t m16 = ((k < 2 ? w0 : w1) >> (16 * (k & 1))) & 0xFFFFu;
-      if (k < nch) process_chunk_masked(r, c0 + 16 * k, Nk, m16, c, st);
+  uint32_t v[32];
+  auto cols = [&](int k) {   // columns 32 k .. 32 k + 31 of the warp's 64
+    if constexpr (kKind == kItemText || kKind == kItemImage) {
+      process_cols_full<kKind == kItemText>(v, c, st);
     } else {
-      process_chunk_full<kKind == kItemText>(r, c, st);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int col0 = c0 + 32 * k + 16 * q;
+        uint32_t r[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) r[e] = v[16 * q + e];
+        if (col0 < Nk) {
+          if (kKind == kItemGeneral)
+            process_chunk(r, col0, Nk, L, c, st);
+          else
+            process_chunk_masked(r, col0, Nk, ((k ? w1 : w0) >> (16 * q)) & 0xFFFFu, c, st);
+        }
+      }
     }
   };
-  tmem_ld16(tb, ra);
-  tmem_wait(ra);
-  tmem_ld16(tb + 16, rb);
-  chunk(ra, 0);
-  tmem_wait(rb);
-  tmem_ld16(tb + 32, ra);
-  chunk(rb, 1);
-  tmem_wait(ra);
-  tmem_ld16(tb + 48, rb);
-  chunk(ra, 2);
-  tmem_wait(rb);
+  tmem_ld32_wait(tb, v);
+  cols(0);
+  tmem_ld32_wait(tb + 32, v);
   fence_before();
   __syncwarp();
   if (lane == 0) mbar_arrive(s_empty);
-  chunk(rb, 3);
+  cols(1);
 }
 
 struct Segment {
@@ -467,7 +469,7 @@ spatial_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   Bars* bars = reinterpret_cast<Bars*>(sK + C::kKBytes);
   float* xch = reinterpret_cast<float*>(bars + 1);   // kXchBytes
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int it_begin = (int)blockIdx.x * p.per;
   const int it_end = min(it_begin + p.per, p.total);
   if (it_begin >= it_end) return;   // block-uniform
@@ -534,69 +536,70 @@ spatial_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 
   if (warp == 0) {
     // ------------------------------------------------------ TMA producer --
-    if (lane == 0) {
-      bool ok = true;
-      int li = 0;
-      int sg = 0;
-      int q_armed = 0;   // Q tiles armed in the latest segment
-      for (int it = it_begin; it < it_end && ok;) {
-        const Segment seg = segment_at(it, it_end, p.n_kt);
-        const int bh = seg.u / p.n_qp, qp = seg.u - bh * p.n_qp;
-        const int b = bh / p.H, h = bh - b * p.H;
-        // the Q buffer is free at the start; later segments wait for the
-        // MMAs of the previous one
-        if (sg > 0) ok = mbar_wait_bounded(&bars->q_empty, (uint32_t)((sg & 1) ^ 1), abort_flag, p.status);
-        if (!ok) break;
-        const bool first = (sg == 0);   // Q tiles and K tile 0 already issued
-        ++sg;   // Q of this segment is being issued
-        q_armed = first ? kQTiles : 0;
-        for (int j = 0; j < seg.nk; ++j, ++li) {
-          // Q tile 0 before the first K tile, Q tile 1 right after it
-          if (!first && (j == 0 || (j == 1 && kQTiles > 1))) {
-            const int t = j;
-            ++q_armed;
-            mbar_arrive_expect_tx(&bars->q_full[t], C::kTileBytes);
-            for (int cb = 0; cb < C::kCB; ++cb)
-              tma_load_4d(sQ + t * C::kTileBytes + cb * (kBM * 128), &tmQ, cb * 64,
-                          qp * kUnitRows + t * kBM, h, b, &bars->q_full[t]);
-          }
-          if (li == 1) {
-            // cold start: the first K tile lands before the rest of the ring
-            // is requested, so the first MMAs do not wait behind every
-            // CTA's whole prologue in HBM
-            ok = mbar_wait_bounded(&bars->k_full[0], 0, abort_flag, p.status);
-            if (!ok) break;
-          }
-          if (li == 0) continue;   // K tile 0 went out before the set-up
-          const int stage = (int)(li % C::kStages);
-          const uint32_t ph = (uint32_t)((li / C::kStages) & 1);
-          ok = mbar_wait_bounded(&bars->k_empty[stage], ph ^ 1u, abort_flag, p.status);
+    bool ok = true;
+    int li = 0;
+    int sg = 0;
+    int q_armed = 0;   // Q tiles armed in the latest segment
+    for (int it = it_begin; it < it_end && ok;) {
+      const Segment seg = segment_at(it, it_end, p.n_kt);
+      const int bh = seg.u / p.n_qp, qp = seg.u - bh * p.n_qp;
+      const int b = bh / p.H, h = bh - b * p.H;
+      auto load_q = [&](int t) {
+        ++q_armed;
+        if (elect_one()) {
+          mbar_arrive_expect_tx(&bars->q_full[t], C::kTileBytes);
+          for (int cb = 0; cb < C::kCB; ++cb)
+            tma_load_4d(sQ + t * C::kTileBytes + cb * (kBM * 128), &tmQ, cb * 64,
+                        qp * kUnitRows + t * kBM, h, b, &bars->q_full[t]);
+        }
+        __syncwarp();
+      };
+      // the Q buffer is free at the start; later segments wait for the
+      // MMAs of the previous one
+      if (sg > 0) ok = mbar_wait_bounded(&bars->q_empty, (uint32_t)((sg & 1) ^ 1), abort_flag, p.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      const bool first = (sg == 0);   // Q tiles and K tile 0 already issued
+      ++sg;   // Q of this segment is being issued
+      q_armed = first ? kQTiles : 0;
+      for (int j = 0; j < seg.nk; ++j, ++li) {
+        // Q tile 0 before the first K tile, Q tile 1 right after it
+        if (!first && j < kQTiles) load_q(j);
+        if (li == 1) {
+          // cold start: the first K tile lands before the rest of the ring
+          // is requested, so the first MMAs do not wait behind every
+          // CTA's whole prologue in HBM
+          ok = mbar_wait_bounded(&bars->k_full[0], 0, abort_flag, p.status);
+          ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
+        }
+        if (li == 0) continue;   // K tile 0 went out before the set-up
+        const int stage = (int)(li % C::kStages);
+        const uint32_t ph = (uint32_t)((li / C::kStages) & 1);
+        ok = mbar_wait_bounded(&bars->k_empty[stage], ph ^ 1u, abort_flag, p.status);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (elect_one()) {
           mbar_arrive_expect_tx(&bars->k_full[stage], C::kTileBytes);
           for (int cb = 0; cb < C::kCB; ++cb)
             tma_load_4d(sK + stage * C::kTileBytes + cb * (kBM * 128), &tmK, cb * 64,
                         (seg.kt0 + j) * kBN, h, b, &bars->k_full[stage]);
         }
-        if (ok && seg.nk == 1 && !first) {   // a one-tile segment still needs Q tile 1
-          ++q_armed;
-          mbar_arrive_expect_tx(&bars->q_full[1], C::kTileBytes);
-          for (int cb = 0; cb < C::kCB; ++cb)
-            tma_load_4d(sQ + C::kTileBytes + cb * (kBM * 128), &tmQ, cb * 64,
-                        qp * kUnitRows + kBM, h, b, &bars->q_full[1]);
-        }
-        it += seg.nk;
+        __syncwarp();
       }
-      if (!ok) {
-        // drain the copies still in flight before the CTA exits: the Q tiles
-        // of the last segment started, then every armed K stage
-        for (int t = 0; t < q_armed; ++t)
-          mbar_wait_bounded(&bars->q_full[t], (uint32_t)((sg - 1) & 1), nullptr, p.status);
-        for (int s = 0; s < C::kStages; ++s) {
-          const int armed = li - s;   // items issued on stage s: li - s > 0
-          if (armed > 0) {
-            const int last = (armed - 1) / C::kStages;
-            mbar_wait_bounded(&bars->k_full[s], (uint32_t)(last & 1), nullptr, p.status);
-          }
+      if (ok && seg.nk == 1 && !first) load_q(1);   // a one-tile segment still needs Q tile 1
+      it += seg.nk;
+    }
+    if (!ok) {
+      // drain the copies still in flight before the CTA exits: the Q tiles
+      // of the last segment started, then every armed K stage
+      for (int t = 0; t < q_armed; ++t)
+        mbar_wait_bounded(&bars->q_full[t], (uint32_t)((sg - 1) & 1), nullptr, p.status);
+      for (int s = 0; s < C::kStages; ++s) {
+        const int armed = li - s;   // items issued on stage s: li - s > 0
+        if (armed > 0) {
+          const int last = (armed - 1) / C::kStages;
+          mbar_wait_bounded(&bars->k_full[s], (uint32_t)(last & 1), nullptr, p.status);
         }
       }
     }
@@ -606,35 +609,34 @@ spatial_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     // stalls that thread's queue of MMAs until the tensor pipe has taken it;
     // with two issuers the other queue keeps the pipe busy meanwhile.
     const int t = (warp == 1) ? 0 : 1;
-    if (lane == 0) {
-      bool ok = true;
-      int li = 0;
-      int sg = 0;
-      // operand descriptors computed once; per MMA only constant offsets are
-      // added (the issuing thread shares its sub-partition with four busy
-      // softmax warps, so every instruction it needs delays the MMAs)
-      const uint32_t a_lo = sw128_desc_lo(sQ + t * C::kTileBytes);
-      const uint32_t b_lo0 = sw128_desc_lo(sK);
-      const uint32_t d_hi = sw128_desc_hi();
-      const uint32_t d_base = tmem + (uint32_t)(t * 2 * kBN);
-      for (int it = it_begin; it < it_end && ok;) {
-        const Segment seg = segment_at(it, it_end, p.n_kt);
-        for (int j = 0; j < seg.nk && ok; ++j, ++li) {
-          const int stage = (int)(li % C::kStages);
-          const uint32_t ph = (uint32_t)((li / C::kStages) & 1);
-          const int sb = (int)(li & 1);
-          const uint32_t sph = (uint32_t)((li >> 1) & 1);
-          ok = mbar_wait_bounded(&bars->k_full[stage], ph, abort_flag, p.status);
-          if (!ok) break;
-          if (j == 0) {
-            ok = mbar_wait_bounded(&bars->q_full[t], (uint32_t)(sg & 1), abort_flag, p.status);
-            if (!ok) break;
-          }
+    bool ok = true;
+    int li = 0;
+    int sg = 0;
+    // operand descriptors computed once; per MMA only constant offsets are
+    // added (the issuing thread shares its sub-partition with four busy
+    // softmax warps, so every instruction it needs delays the MMAs)
+    const uint32_t a_lo = sw128_desc_lo(sQ + t * C::kTileBytes);
+    const uint32_t b_lo0 = sw128_desc_lo(sK);
+    const uint32_t d_hi = sw128_desc_hi();
+    const uint32_t d_base = tmem + (uint32_t)(t * 2 * kBN);
+    for (int it = it_begin; it < it_end && ok;) {
+      const Segment seg = segment_at(it, it_end, p.n_kt);
+      for (int j = 0; j < seg.nk && ok; ++j, ++li) {
+        const int stage = (int)(li % C::kStages);
+        const uint32_t ph = (uint32_t)((li / C::kStages) & 1);
+        const int sb = (int)(li & 1);
+        const uint32_t sph = (uint32_t)((li >> 1) & 1);
+        ok = mbar_wait_bounded(&bars->k_full[stage], ph, abort_flag, p.status);
+        if (ok && j == 0)
+          ok = mbar_wait_bounded(&bars->q_full[t], (uint32_t)(sg & 1), abort_flag, p.status);
+        if (ok)
           ok = mbar_wait_bounded(&bars->s_empty[t][sb], sph ^ 1u, abort_flag, p.status);
-          if (!ok) break;
-          fence_after();
-          const uint32_t d_tmem = d_base + (uint32_t)(sb * kBN);
-          const uint32_t b_lo = b_lo0 + (uint32_t)((stage * C::kTileBytes) >> 4);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        fence_after();
+        const uint32_t d_tmem = d_base + (uint32_t)(sb * kBN);
+        const uint32_t b_lo = b_lo0 + (uint32_t)((stage * C::kTileBytes) >> 4);
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk) {
             const uint32_t off = (uint32_t)(((kk >> 2) * (kBM * 128) + (kk & 3) * 32) >> 4);
@@ -642,16 +644,17 @@ spatial_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           }
           mma_commit(&bars->s_full[t][sb]);
           mma_commit(&bars->k_empty[stage]);
+          if (j == seg.nk - 1) mma_commit(&bars->q_empty);
         }
-        if (!ok) break;
-        mma_commit(&bars->q_empty);
-        it += seg.nk;
-        ++sg;
+        __syncwarp();
       }
-      // all issued MMAs complete before tensor memory is released
-      mma_commit(&bars->drain[t]);
-      mbar_wait_bounded(&bars->drain[t], 0, nullptr, p.status);
+      it += seg.nk;
+      ++sg;
     }
+    // all issued MMAs complete before tensor memory is released
+    if (elect_one()) mma_commit(&bars->drain[t]);
+    __syncwarp();
+    mbar_wait_bounded(&bars->drain[t], 0, nullptr, p.status);
   } else {
     // ---------------------------------------------------- softmax-reduce --
     const int g = (warp - 2) >> 2;        // warpgroup: query tile t, column half ch

@@ -11,6 +11,18 @@
 namespace avits {
 namespace tc {
 
+// One lane of a converged warp.  Code under it is known to the compiler to be
+// single-threaded, so the operands that tcgen05.mma and the TMA copies take in
+// uniform registers are moved there once; under `lane == 0` every instruction
+// pays for a possibly divergent value.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 // ------------------------------------------------------------------- TMA ---
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int c0, int c1,
                                             int c2, int c3, uint64_t* bar) {
@@ -157,6 +169,24 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
       "%28, %29, %30, %31}, [%32];"
       : AVITS_R8(0), AVITS_R8(8), AVITS_R8(16), AVITS_R8(24)
       : "r"(taddr));
+}
+
+#define AVITS_O8(r, b) "=r"(r[b]), "=r"(r[b + 1]), "=r"(r[b + 2]), "=r"(r[b + 3]), \
+                       "=r"(r[b + 4]), "=r"(r[b + 5]), "=r"(r[b + 6]), "=r"(r[b + 7])
+
+// Loads with the wait in the same statement, for the softmax loops: a separate
+// wait has to name the registers as in-out operands to keep their uses behind
+// it, and the compiler then copied them (4 % of the spatial kernel's time).
+// 32 consecutive columns, complete on return.
+__device__ __forceinline__ void tmem_ld32_wait(uint32_t taddr, uint32_t (&a)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+      "%11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
+      "%28, %29, %30, %31}, [%32];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : AVITS_O8(a, 0), AVITS_O8(a, 8), AVITS_O8(a, 16), AVITS_O8(a, 24)
+      : "r"(taddr)
+      : "memory");
 }
 
 // Completes the thread's outstanding tcgen05.ld; the registers are tied to
