@@ -308,20 +308,32 @@ __device__ __forceinline__ float vec_elem<__nv_bfloat16>(const uint4& v, int e) 
 }
 
 // 16-byte vectors of kE elements; kNT >= n_t snapshots kept in registers.
+// kLanes threads per token: all 128 of the CTA for rows of 128 vectors and more
+// (D = 3072 bf16: three vectors per thread, then one barrier; 6.46 TB/s), a
+// warp below that, part of one for rows of up to 16 vectors, so that few
+// threads are without a vector and no token waits at a barrier.  With a CTA
+// per token throughout, us before -> now: D = 128 bf16, 2 snapshots, 65536
+// tokens 59.6 -> 12.4, 16384 tokens 13.6 -> 4.0; D = 768, 3 snapshots, 16384
+// tokens 21.0 -> 15.2 (1024 tokens 2.8 -> 2.9); D = 128 fp32, 4 snapshots,
+// 16384 tokens 16.0 -> 7.4.
 constexpr int kVarThreads = 128;
 
-template <typename T, int kNT>
+template <typename T, int kNT, int kLanes>
 __global__ void __launch_bounds__(kVarThreads)
 temporal_var_vec_kernel(SnapPtrs snaps, int n_t, int64_t ntok, int D, float* __restrict__ V) {
   constexpr int kE = 16 / (int)sizeof(T);
+  constexpr int kTokens = kVarThreads / kLanes;   // per CTA
   __shared__ float part[kVarThreads / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int gl = threadIdx.x % kLanes;
   const int nv = D / kE;
   const float inv_n = 1.0f / (float)n_t;
   const float inv_n1 = 1.0f / (float)(n_t - 1);
-  for (int64_t t = blockIdx.x; t < ntok; t += gridDim.x) {
+  // every thread of the CTA runs the same number of rounds
+  for (int64_t t0 = (int64_t)blockIdx.x * kTokens; t0 < ntok; t0 += (int64_t)gridDim.x * kTokens) {
+    const int64_t t = t0 + threadIdx.x / kLanes;
     float acc = 0.f;
-    for (int v = threadIdx.x; v < nv; v += kVarThreads) {
+    for (int v = t < ntok ? gl : nv; v < nv; v += kLanes) {
       uint4 raw[kNT];
 #pragma unroll
       for (int s = 0; s < kNT; ++s)
@@ -351,17 +363,45 @@ temporal_var_vec_kernel(SnapPtrs snaps, int n_t, int64_t ntok, int D, float* __r
         acc += ss * inv_n1;
       }
     }
-    acc = warp_sum(acc);
-    if (lane == 0) part[w] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float tot = 0.f;
 #pragma unroll
-      for (int k = 0; k < kVarThreads / 32; ++k) tot += part[k];
-      V[t] = tot / (float)D;
+    for (int o = (kLanes < 32 ? kLanes : 32) / 2; o > 0; o >>= 1)
+      acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if constexpr (kLanes <= 32) {
+      if (gl == 0 && t < ntok) V[t] = acc / (float)D;
+    } else {
+      if (lane == 0) part[w] = acc;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        float tot = 0.f;
+#pragma unroll
+        for (int k = 0; k < kVarThreads / 32; ++k) tot += part[k];
+        V[t] = tot / (float)D;
+      }
+      __syncthreads();   // part[] is reused by the next token
     }
-    __syncthreads();   // part[] is reused by the next token
   }
+}
+
+template <typename T, int kNT>
+void launch_var_lanes(const SnapPtrs& sp, int n_t, int64_t ntok, int D, float* V, cudaStream_t s) {
+  const int nv = D * (int)sizeof(T) / 16;
+  const int lanes = nv <= 8 ? 8 : nv <= 16 ? 16 : nv < kVarThreads ? 32 : kVarThreads;
+  // a plain launch: as a programmatic dependent the waiting CTAs took SM slots
+  // from the kernel before and measured slower (grid-stride beyond 2^31 - 1)
+  const int per = kVarThreads / lanes;
+  const unsigned grid = (unsigned)std::min<int64_t>((ntok + per - 1) / per, (int64_t)INT32_MAX);
+  auto kern = lanes == 8    ? temporal_var_vec_kernel<T, kNT, 8>
+              : lanes == 16 ? temporal_var_vec_kernel<T, kNT, 16>
+              : lanes == 32 ? temporal_var_vec_kernel<T, kNT, 32>
+                            : temporal_var_vec_kernel<T, kNT, kVarThreads>;
+  kern<<<grid, kVarThreads, 0, s>>>(sp, n_t, ntok, D, V);
+}
+
+template <typename T>
+void launch_var_vec(const SnapPtrs& sp, int n_t, int64_t ntok, int D, float* V, cudaStream_t s) {
+  if (n_t <= 4) launch_var_lanes<T, 4>(sp, n_t, ntok, D, V, s);
+  else if (n_t <= 8) launch_var_lanes<T, 8>(sp, n_t, ntok, D, V, s);
+  else launch_var_lanes<T, kMaxSnapshots>(sp, n_t, ntok, D, V, s);
 }
 
 }  // namespace
@@ -482,26 +522,8 @@ cudaError_t launch_temporal_var(const void* const* snaps, int n_t, avits_dtype d
   bool vec = ((int64_t)D * elt) % 16 == 0;
   for (int i = 0; i < n_t; ++i) vec = vec && (reinterpret_cast<uintptr_t>(snaps[i]) & 15u) == 0;
   if (vec) {
-    // one CTA per token (grid-stride beyond 2^31 - 1 tokens).  A plain
-    // launch: as a programmatic dependent its waiting CTAs took SM slots from
-    // the kernel before it and measured slower.
-    const unsigned grid = (unsigned)std::min<int64_t>(ntok, (int64_t)INT32_MAX);
-    if (dt == AVITS_BF16) {
-      if (n_t <= 4)
-        temporal_var_vec_kernel<__nv_bfloat16, 4><<<grid, kVarThreads, 0, s>>>(sp, n_t, ntok, D, V);
-      else if (n_t <= 8)
-        temporal_var_vec_kernel<__nv_bfloat16, 8><<<grid, kVarThreads, 0, s>>>(sp, n_t, ntok, D, V);
-      else
-        temporal_var_vec_kernel<__nv_bfloat16, kMaxSnapshots>
-            <<<grid, kVarThreads, 0, s>>>(sp, n_t, ntok, D, V);
-    } else {
-      if (n_t <= 4)
-        temporal_var_vec_kernel<float, 4><<<grid, kVarThreads, 0, s>>>(sp, n_t, ntok, D, V);
-      else if (n_t <= 8)
-        temporal_var_vec_kernel<float, 8><<<grid, kVarThreads, 0, s>>>(sp, n_t, ntok, D, V);
-      else
-        temporal_var_vec_kernel<float, kMaxSnapshots><<<grid, kVarThreads, 0, s>>>(sp, n_t, ntok, D, V);
-    }
+    if (dt == AVITS_BF16) launch_var_vec<__nv_bfloat16>(sp, n_t, ntok, D, V, s);
+    else launch_var_vec<float>(sp, n_t, ntok, D, V, s);
     return cudaGetLastError();
   }
   const int grid = grid_for(ntok, num_sms);
