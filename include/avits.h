@@ -436,8 +436,8 @@ avits_status avits_select_upsample(const float* A, const float* V, const float* 
  * out_full : [B,full_h*full_w,C*4] same dtype.
  * workspace : avits_merge_final_workspace() bytes (both modes), 16-byte
  *             aligned, ZERO-FILLED before its first use; the calls keep it
- *             consistent afterwards (nearest: a claim map tagged per call and
- *             a counter each call clears; bilinear: a cell map it refills).
+ *             consistent afterwards (a counter each call clears and a map of
+ *             the cells whose old entries no call takes for its own).
  * ---------------------------------------------------------------------- */
 avits_status avits_merge_final(const void* mixed, avits_dtype dt, int B, int N,
                                const int32_t* pos, const int32_t* span, int full_h, int full_w,

@@ -174,6 +174,55 @@ struct Pix4<__nv_bfloat16> {
   }
 };
 
+// The 16 bytes of one token that hold kCh channels, as pixels.
+template <typename T>
+struct Chunk;
+template <>
+struct Chunk<float> {
+  static constexpr int kCh = 1;
+  __device__ static void unpack(const uint4& w, float (&p)[1][4]) {
+    p[0][0] = __uint_as_float(w.x); p[0][1] = __uint_as_float(w.y);
+    p[0][2] = __uint_as_float(w.z); p[0][3] = __uint_as_float(w.w);
+  }
+  __device__ static uint4 pack(const float (&p)[1][4]) {
+    return make_uint4(__float_as_uint(p[0][0]), __float_as_uint(p[0][1]),
+                      __float_as_uint(p[0][2]), __float_as_uint(p[0][3]));
+  }
+};
+template <>
+struct Chunk<__nv_bfloat16> {
+  static constexpr int kCh = 2;
+  __device__ static void unpack(const uint4& w, float (&p)[2][4]) {
+    p[0][0] = bf16_lo(w.x); p[0][1] = bf16_hi(w.x); p[0][2] = bf16_lo(w.y); p[0][3] = bf16_hi(w.y);
+    p[1][0] = bf16_lo(w.z); p[1][1] = bf16_hi(w.z); p[1][2] = bf16_lo(w.w); p[1][3] = bf16_hi(w.w);
+  }
+  __device__ static uint4 pack(const float (&p)[2][4]) {
+    const uint2 a = Pix4<__nv_bfloat16>::make(p[0][0], p[0][1], p[0][2], p[0][3]);
+    const uint2 b = Pix4<__nv_bfloat16>::make(p[1][0], p[1][1], p[1][2], p[1][3]);
+    return make_uint4(a.x, a.y, b.x, b.y);
+  }
+};
+
+// The 16 bytes of a token with every channel's pixels taken from (r0|r1,
+// c0|c1): pixel (0,0) <- (r0,c0), (0,1) <- (r0,c1), (1,0) <- (r1,c0), (1,1) <-
+// (r1,c1).
+template <typename T>
+__device__ __forceinline__ uint4 select_pixels(const uint4& w, int r0, int r1, int c0, int c1);
+template <>
+__device__ __forceinline__ uint4 select_pixels<float>(const uint4& w, int r0, int r1, int c0,
+                                                      int c1) {
+  auto at = [&](int r, int c) { return r ? (c ? w.w : w.z) : (c ? w.y : w.x); };
+  return make_uint4(at(r0, c0), at(r0, c1), at(r1, c0), at(r1, c1));
+}
+template <>
+__device__ __forceinline__ uint4 select_pixels<__nv_bfloat16>(const uint4& w, int r0, int r1,
+                                                              int c0, int c1) {
+  // a channel is two words, row 0 and row 1, column 0 in the low half
+  const unsigned sel = (c0 ? 0x32u : 0x10u) | (c1 ? 0x3200u : 0x1000u);
+  return make_uint4(__byte_perm(r0 ? w.y : w.x, 0u, sel), __byte_perm(r1 ? w.y : w.x, 0u, sel),
+                    __byte_perm(r0 ? w.w : w.z, 0u, sel), __byte_perm(r1 ? w.w : w.z, 0u, sel));
+}
+
 // One 16-byte chunk j of a latent token (channel, patch row, patch column
 // layout) whose channel pixels are taken from a source token's pixels
 // (r0|r1, c0|c1): pixel (0,0) <- (r0,c0), (0,1) <- (r0,c1), (1,0) <- (r1,c0),

@@ -2,19 +2,23 @@
 // Stage 3: the remaining tokens are expanded and the sequence is laid out in
 // spatial order).
 //
-// Nearest: one warp per mixed token scatters its s x s cells; full-res pixel
-// (Y,X) of a token at (y,x) with span s takes token pixel ((Y-2y)/s, (X-2x)/s).
-// Coverage is checked in the same kernel: every cell is claimed by an
-// atomicExch of this call's tag into a claim map in the caller's workspace
-// (an old value equal to the tag = a cell covered twice), and every CTA adds
-// (1 << 40) | cells claimed to one 64-bit word; the CTA whose add completes
-// the CTA count compares the claimed total with B * fh * fw (fewer = a hole,
-// since no cell was claimed twice), clears the word and advances the tag
-// for the next call.  The map needs no clearing between calls.
-// Bilinear (spans 1, 2 and 4): a cell map is scattered first (atomicExch into
-// a -1-filled workspace, so double cover and holes are detected), then every
-// output (cell, channel) gathers: span-1 cells are copied, coarser cells take
-// the half-pixel-centred 2x bilinear resize of level 1 of the frame's pixel
+// Nearest: full-res pixel (Y,X) of a token at (y,x) with span s takes token
+// pixel ((Y-2y)/s, (X-2x)/s).  Few tokens (a batch of one): one warp per token
+// writes its s x s cells in one pass; every cell is claimed by an atomicExch of
+// this call's tag into a claim map in the caller's workspace (an old value equal
+// to the tag = a cell covered twice).  More tokens: pass 1 writes each token's
+// index into the words of its cells with plain stores, pass 2 goes over the
+// cells and takes a word only if that token covers the cell in this call, so an
+// entry of an earlier call is no cover.  One pass waits for a chain of round
+// trips per token and for an atomic per cell; two passes are streams.
+// Either way every CTA of the counting kernel adds (1 << 40) | cells to one
+// 64-bit word, and the CTA whose add completes the CTA count compares the total
+// with B * fh * fw (in two passes a cell covered twice makes it differ, or
+// leaves a hole that pass 2 finds), then clears the word.  The map needs no
+// clearing between calls.
+// Bilinear (spans 1, 2 and 4): pass 1 as above with each entry carrying the
+// token's level; in pass 2 span-1 cells are copied, coarser cells take the
+// half-pixel-centred 2x bilinear resize of level 1 of the frame's pixel
 // pyramid (frame_map.cuh), refined first from level 2 inside span-4 tokens.
 // Algorithmic bytes: B*N*(T*elt + 12) read + B*fh*fw*T*elt written.
 #include <algorithm>
@@ -27,8 +31,8 @@ namespace avits {
 namespace {
 
 // Workspace of the merge: a 16-byte header, then one 32-bit word per output
-// cell.  Nearest: header = (tag of the last call, unused, 64-bit CTA count |
-// claimed cells), words = claim map.  Bilinear: the words are the cell map.
+// cell.  Header = (tag of the last one-pass call, unused, 64-bit CTA count |
+// cells), words = claim map (one pass) or cell map (two passes, bilinear).
 struct MergeHeader {
   uint32_t last_tag;
   uint32_t unused;
@@ -36,16 +40,26 @@ struct MergeHeader {
 };
 constexpr int kMergeHeaderBytes = 16;
 
-// Claim tags have bit 31 set (bilinear cell-map entries, -1 aside, have it
-// clear, so a workspace used in both modes never confuses the two) and a
+// Claim tags have bit 31 set (token indices and cell-map entries, -1 aside, have
+// it clear, so a workspace used in both modes never confuses the two) and a
 // 31-bit call counter in 1 .. 2^31 - 2 (never 0, the zeroed map).
 __device__ __forceinline__ uint32_t next_tag(uint32_t last) {
   const uint32_t g = last & 0x7FFFFFFFu;
   return 0x80000000u | ((g == 0u || g >= 0x7FFFFFFEu) ? 1u : g + 1u);
 }
 
-// Batch-1 sized inputs (at most one token per warp of a capped grid): one
-// warp per token, one pass.  A token's area is known once its position and
+// A CTA has written `cells` cells; the CTA that completes the count compares
+// the total with the frame's and clears the word for the next call.
+__device__ __forceinline__ void count_cells(MergeHeader* hdr, unsigned long long cells,
+                                            unsigned long long frame, unsigned int* status) {
+  const unsigned long long mine = (1ull << 40) | cells;
+  const unsigned long long v = atomicAdd(&hdr->count, mine) + mine;
+  if ((v >> 40) != (unsigned long long)gridDim.x) return;
+  if ((v & ((1ull << 40) - 1ull)) != frame) raise_status(status, AVITS_ERR_COVERAGE);
+  hdr->count = 0ull;
+}
+
+// Few tokens: one warp per token, one pass.  A token's area is known once its position and
 // span are read, so the CTA's count goes out first; the claims, the count's
 // atomic and the pixel loads are then in flight together and their results
 // are examined last: the check adds no round trip to the copy's two
@@ -141,138 +155,122 @@ merge_nearest_warp_kernel(const T* __restrict__ mixed, int B, int N,
   if (twice || old0 == tag || old1 == tag) raise_status(status, AVITS_ERR_COVERAGE);
 }
 
-// Large batches: kLanesPerTok (8) lanes per token (8 x 16 bytes = a
-// 16-channel bf16 token), four tokens in flight per warp; kNearestWarps warps
-// per CTA, at most
-// kNearestCtasPerSm CTAs per SM looping over the tokens (every CTA adds to
-// the one count word, and same-address atomics are serialised: one CTA per
-// 8 tokens of a batch of 64 made the count the bound).  A token's area is
-// known once its position and span are read, so pass 1 sums the CTA's
-// areas and its count goes out before pass 2 copies; the claims, the
-// count's atomic and the pixel loads are then in flight together and their
-// results are examined last.  The first token of each lane group keeps its
-// position in registers between the passes (at batch 1 that is its only
-// token).
-constexpr int kNearestWarps = 8;
-constexpr int kNearestCtasPerSm = 4;
-constexpr int kStageBytes = 512;   // per token slot: a token of up to 512 B takes the vector path
-
-template <typename T, int kLanesPerTok>
-__global__ void __launch_bounds__(kNearestWarps * 32)
-merge_nearest_kernel(const T* __restrict__ mixed, int B, int N, const int32_t* __restrict__ pos,
-                     const int32_t* __restrict__ span, int fh, int fw, int C, T* __restrict__ out,
-                     MergeHeader* hdr, uint32_t* __restrict__ claim, unsigned int* status) {
-  using PV = typename Pix4<T>::V;
-  constexpr int kToksPerWarp = 32 / kLanesPerTok;
+// Large batches, pass 1: as merge_scatter_kernel below, for tokens of any span
+// and position; the word of a cell is the token's index.  A token of more than
+// 16 cells is written by its whole warp.
+__global__ void __launch_bounds__(256)
+merge_index_kernel(int B, int N, const int32_t* __restrict__ pos, const int32_t* __restrict__ span,
+                   int fh, int fw, int32_t* __restrict__ map, MergeHeader* hdr,
+                   unsigned int* status) {
   pdl_wait_then_trigger();
-  __shared__ __align__(16) uint8_t stage_all[kNearestWarps * kToksPerWarp * kStageBytes];
-  __shared__ unsigned int cta_cells;
-  if (threadIdx.x == 0) cta_cells = 0u;
-  const uint32_t last = *reinterpret_cast<volatile uint32_t*>(&hdr->last_tag);
-  const int lane = threadIdx.x & 31, grp = lane / kLanesPerTok, gl = lane % kLanesPerTok;
-  const int warp = threadIdx.x >> 5;
-  const int64_t ntok = (int64_t)B * N;
-  const int64_t tstride = (int64_t)gridDim.x * kNearestWarps * kToksPerWarp;
-  const int64_t t0 = ((int64_t)blockIdx.x * kNearestWarps + warp) * kToksPerWarp + grp;
-  // pass 1: validate the tokens and sum their areas
-  unsigned int cells = 0u;
-  int y0 = 0, x0 = 0, s0 = 0;
-  for (int64_t t = t0; t < ntok; t += tstride) {
-    const int y = pos[t * 2], x = pos[t * 2 + 1], sp = span[t];
-    if (t == t0) { y0 = y; x0 = x; s0 = sp; }
-    if (sp <= 0 || y < 0 || x < 0 || y + sp > fh || x + sp > fw) {
-      if (gl == 0) raise_status(status, AVITS_ERR_COVERAGE);
-    } else if (gl == 0) {
-      cells += (unsigned int)(sp * sp);
-    }
-  }
-  __syncthreads();   // cta_cells is initialised
-  if (cells) atomicAdd(&cta_cells, cells);
+  __shared__ unsigned long long cta_cells;
+  if (threadIdx.x == 0) cta_cells = 0ull;
   __syncthreads();
-  unsigned long long v = 0ull;
-  if (threadIdx.x == 0)
-    v = atomicAdd(&hdr->count, (1ull << 40) | (unsigned long long)cta_cells) +
-        ((1ull << 40) | (unsigned long long)cta_cells);
-  const uint32_t tag = next_tag(last);
-  bool twice = false;
-  uint8_t* stage = stage_all + (warp * kToksPerWarp + grp) * kStageBytes;
-  const int T4 = C * 4;
-  const int tb = T4 * (int)sizeof(T);
-  const bool vec = (tb & 15) == 0 && tb <= kStageBytes;
-  // pass 2: claim the cells and copy (all lanes of the warp run the same
-  // number of iterations, so the warp-wide syncs below are safe)
-  const int64_t iters = (ntok - (t0 - grp) + tstride - 1) / tstride;
-  for (int64_t it = 0; it < iters; ++it) {
-    const int64_t t = t0 + it * tstride;
-    const bool have = t < ntok;
-    int y = 0, x = 0, sp = 0;
-    if (have) {
-      if (it == 0) { y = y0; x = x0; sp = s0; }
-      else { y = pos[t * 2]; x = pos[t * 2 + 1]; sp = span[t]; }
-    }
-    const bool ok = have && !(sp <= 0 || y < 0 || x < 0 || y + sp > fh || x + sp > fw);
-    const T* src = mixed + (have ? t : 0) * T4;
-    if (vec) {
-      __syncwarp();   // the slot's previous token is read
-      if (ok)
-        for (int q = gl; q < tb / 16; q += kLanesPerTok)
-          reinterpret_cast<uint4*>(stage)[q] = __ldg(reinterpret_cast<const uint4*>(src) + q);
-      __syncwarp();
-    }
-    if (!ok) continue;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  int y = 0, x = 0, s = 0, ti = 0;
+  int64_t base = 0;
+  if (t < (int64_t)B * N) {
     const int b = (int)(t / N);
-    const int64_t base = (int64_t)b * fh * fw;
-    const int area = sp * sp;
-    // claims of cells gl and gl + kLanesPerTok are examined after the copy,
-    // so their round trip overlaps it
-    uint32_t old0 = 0u, old1 = 0u;
-    if (gl < area)
-      old0 = atomicExch(&claim[base + (int64_t)(y + gl / sp) * fw + (x + gl % sp)], tag);
-    if (gl + kLanesPerTok < area) {
-      const int c1 = gl + kLanesPerTok;
-      old1 = atomicExch(&claim[base + (int64_t)(y + c1 / sp) * fw + (x + c1 % sp)], tag);
-    }
-    for (int cell = gl + 2 * kLanesPerTok; cell < area; cell += kLanesPerTok)
-      twice |= atomicExch(&claim[base + (int64_t)(y + cell / sp) * fw + (x + cell % sp)], tag) == tag;
-    if (vec) {
-      // 16-byte output chunks: cell (u, w) of the token's s x s block takes,
-      // for channel c, the token's pixels (r0|r1, c0|c1); chunks of one cell
-      // are consecutive, so the stores are coalesced
-      const int cpc = tb / 16;
-      for (int q = gl; q < area * cpc; q += kLanesPerTok) {
-        const int cell = q / cpc, j = q - cell * cpc;
-        const int u = cell / sp, w = cell - u * sp;
-        const int r0 = (2 * u) / sp, r1 = (2 * u + 1) / sp;
-        const int c0 = (2 * w) / sp, c1 = (2 * w + 1) / sp;
-        const uint4 chunk = (sp == 1) ? reinterpret_cast<const uint4*>(stage)[j]
-                                      : gather_chunk<T>(stage, j, r0, r1, c0, c1);
-        const int64_t ocell = base + (int64_t)(y + u) * fw + (x + w);
-        reinterpret_cast<uint4*>(out + ocell * T4)[j] = chunk;
-      }
-    } else {
-      for (int task = gl; task < area * C; task += kLanesPerTok) {
-        const int cell = task / C, c = task - cell * C;
-        const int u = cell / sp, w = cell - u * sp;
-        const int r0 = (2 * u) / sp, r1 = (2 * u + 1) / sp;
-        const int c0 = (2 * w) / sp, c1 = (2 * w + 1) / sp;
-        const T* sc = src + c * 4;
-        const float p00 = load_elem(sc, r0 * 2 + c0), p01 = load_elem(sc, r0 * 2 + c1);
-        const float p10 = load_elem(sc, r1 * 2 + c0), p11 = load_elem(sc, r1 * 2 + c1);
-        const int64_t ocell = base + (int64_t)(y + u) * fw + (x + w);
-        reinterpret_cast<PV*>(out + ocell * T4)[c] = Pix4<T>::make(p00, p01, p10, p11);
-      }
-    }
-    twice |= old0 == tag || old1 == tag;
-  }
-  if (threadIdx.x == 0 && (v >> 40) == (unsigned long long)gridDim.x) {
-    // every CTA has counted its cells: no cell is claimed twice unless that
-    // is reported, so fewer claimed cells than cells means a hole
-    if ((v & ((1ull << 40) - 1ull)) != (unsigned long long)B * fh * fw)
+    ti = (int)(t - (int64_t)b * N);
+    y = pos[t * 2];
+    x = pos[t * 2 + 1];
+    s = span[t];
+    base = (int64_t)b * fh * fw;
+    if (s <= 0 || y < 0 || x < 0 || y + s > fh || x + s > fw) {
       raise_status(status, AVITS_ERR_COVERAGE);
-    hdr->count = 0ull;
-    hdr->last_tag = tag;
+      s = 0;
+    }
   }
-  if (twice) raise_status(status, AVITS_ERR_COVERAGE);   // a cell claimed twice
+  if (s <= 4)
+    for (int u = 0; u < s; ++u)
+      for (int v = 0; v < s; ++v) map[base + (int64_t)(y + u) * fw + x + v] = ti;
+  for (unsigned big = __ballot_sync(0xffffffffu, s > 4); big; big &= big - 1) {
+    const int src = __ffs(big) - 1;
+    const int ys = __shfl_sync(0xffffffffu, y, src), xs = __shfl_sync(0xffffffffu, x, src);
+    const int ss = __shfl_sync(0xffffffffu, s, src), es = __shfl_sync(0xffffffffu, ti, src);
+    const int64_t bs = __shfl_sync(0xffffffffu, base, src);
+    for (int u = 0; u < ss; ++u)
+      for (int v = lane; v < ss; v += 32) map[bs + (int64_t)(ys + u) * fw + xs + v] = es;
+  }
+  unsigned long long cells = (unsigned long long)s * (unsigned long long)s;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) cells += __shfl_xor_sync(0xffffffffu, cells, o);
+  if (lane == 0 && cells) atomicAdd(&cta_cells, cells);
+  __syncthreads();
+  if (threadIdx.x == 0)
+    count_cells(hdr, cta_cells, (unsigned long long)B * fh * fw, status);
+}
+
+// Large batches, pass 2: one thread per (cell, 16-byte piece of a token; one
+// channel where tokens are not whole pieces), kGatherPieces of them per thread,
+// reading and writing neighbouring pieces with neighbouring threads.  A cell
+// whose word is not a token of this call that covers it is a hole: reported and
+// not written.
+constexpr int kGatherPieces = 4;
+
+template <typename T, bool kVec>
+__global__ void __launch_bounds__(256)
+merge_nearest_gather_kernel(const T* __restrict__ mixed, int N, const int32_t* __restrict__ pos,
+                            const int32_t* __restrict__ span, int fh, int fw, int C,
+                            const int32_t* __restrict__ map, T* __restrict__ out,
+                            unsigned int* status, unsigned ctas) {
+  using PV = typename Pix4<T>::V;
+  pdl_wait_then_trigger();
+  const int T4 = C * 4;
+  const unsigned parts = kVec ? (unsigned)(T4 * sizeof(T) / 16) : (unsigned)C;
+  const unsigned cells = (unsigned)fh * (unsigned)fw;
+  const int b = (int)(blockIdx.x / ctas);
+  const unsigned g0 = (blockIdx.x - b * ctas) * (256u * kGatherPieces) + threadIdx.x;
+  const int32_t* mapb = map + (int64_t)b * cells;
+  const int32_t* posb = pos + (int64_t)b * N * 2;
+  const int32_t* spanb = span + (int64_t)b * N;
+  const T* mb = mixed + (int64_t)b * N * T4;
+  unsigned cell[kGatherPieces], j[kGatherPieces];
+  int t[kGatherPieces];
+#pragma unroll
+  for (int k = 0; k < kGatherPieces; ++k) {
+    const unsigned g = g0 + k * 256u;
+    cell[k] = g / parts;
+    j[k] = g - cell[k] * parts;
+    t[k] = cell[k] < cells ? mapb[cell[k]] : -1;
+  }
+  // the token's place and its piece at once: a word that is no token of this
+  // call reads token 0 and is refused below
+  int y[kGatherPieces], x[kGatherPieces], s[kGatherPieces];
+  uint4 in[kGatherPieces];
+#pragma unroll
+  for (int k = 0; k < kGatherPieces; ++k) {
+    if (t[k] >= N) t[k] = -1;
+    const int tt = max(t[k], 0);
+    y[k] = posb[(int64_t)tt * 2];
+    x[k] = posb[(int64_t)tt * 2 + 1];
+    s[k] = spanb[tt];
+    if constexpr (kVec) in[k] = __ldg(reinterpret_cast<const uint4*>(mb + (int64_t)tt * T4) + j[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < kGatherPieces; ++k) {
+    if (cell[k] >= cells) continue;
+    const int Y = (int)(cell[k] / (unsigned)fw), X = (int)(cell[k] % (unsigned)fw);
+    const int u = Y - y[k], w = X - x[k], sp = s[k];
+    if (t[k] < 0 || u < 0 || w < 0 || u >= sp || w >= sp || y[k] < 0 || x[k] < 0 ||
+        y[k] + sp > fh || x[k] + sp > fw) {
+      raise_status(status, AVITS_ERR_COVERAGE);
+      continue;
+    }
+    T* dst = out + ((int64_t)b * cells + cell[k]) * T4;
+    // the token's pixel rows and columns of this cell's two
+    const int r0 = (2 * u >= sp) ? 1 : 0, r1 = (2 * u + 1 >= sp) ? 1 : 0;
+    const int c0 = (2 * w >= sp) ? 1 : 0, c1 = (2 * w + 1 >= sp) ? 1 : 0;
+    if constexpr (kVec) {
+      reinterpret_cast<uint4*>(dst)[j[k]] = sp == 1 ? in[k] : select_pixels<T>(in[k], r0, r1, c0, c1);
+    } else {
+      const T* sc = mb + (int64_t)t[k] * T4 + j[k] * 4;
+      reinterpret_cast<PV*>(dst)[j[k]] =
+          Pix4<T>::make(load_elem(sc, r0 * 2 + c0), load_elem(sc, r0 * 2 + c1),
+                        load_elem(sc, r1 * 2 + c0), load_elem(sc, r1 * 2 + c1));
+    }
+  }
 }
 
 // The cell map starts as -1 everywhere (a hole until a token claims it).
@@ -305,15 +303,111 @@ __global__ void merge_map_kernel(int B, int N, const int32_t* __restrict__ pos,
     }
 }
 
-// One thread per (output cell, channel).  A span-1 cell is copied.  A coarser
-// cell's four pixels are the 2x bilinear resize of level 1 around it (a 3 x 3
-// neighbourhood of level-1 pixels, clamped to the frame), where level 1 is the
-// frame's own pyramid level, or, inside a span-4 token, the 2x bilinear
-// resize of level 2 (the coarse-to-fine cascade; spans are at most 4).
+// The four pixels of a cell from level-1 pixels around it: output pixel row
+// 2Y + a draws on level-1 rows (Y - 1, Y) for a = 0 and (Y, Y + 1) for a = 1
+// with weights (1/4, 3/4) / (3/4, 1/4), clamped at the frame edge by the
+// neighbourhood; columns likewise.  lv[u][v] is the cell's upper left
+// neighbour.
+template <int K>
+__device__ __forceinline__ void resize_cell(const float (&lv)[K][K], int u, int v, float (&r)[4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int a = q >> 1, b = q & 1;
+    r[q] = bil_combine(lv[u + a][v + b], lv[u + a][v + b + 1], lv[u + a + 1][v + b],
+                       lv[u + a + 1][v + b + 1], a ? 0.75f : 0.25f, a ? 0.25f : 0.75f,
+                       b ? 0.75f : 0.25f, b ? 0.25f : 0.75f);
+  }
+}
+
+// Bilinear merge, pass 1.  One thread per token: its s x s cells get
+// map_entry(token, log2 s) by plain stores into a map that still holds the
+// entries of earlier calls; the CTAs add up the cells written as the nearest
+// merge does.  Pass 2 takes an entry only if its token covers the cell, so a
+// cell nothing wrote in this call is found there; a double cover makes the
+// total differ, or leaves such a cell.  That needs neither a fill of the map
+// nor atomics on its cells.
+__global__ void __launch_bounds__(256)
+merge_scatter_kernel(int B, int N, const int32_t* __restrict__ pos,
+                     const int32_t* __restrict__ span, int fh, int fw,
+                     int32_t* __restrict__ map, MergeHeader* hdr, unsigned int* status) {
+  pdl_wait_then_trigger();
+  __shared__ unsigned int cta_cells;
+  if (threadIdx.x == 0) cta_cells = 0u;
+  __syncthreads();
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned int cells = 0u;
+  if (t < (int64_t)B * N) {
+    const int b = (int)(t / N), ti = (int)(t - (int64_t)b * N);
+    const int y = pos[t * 2], x = pos[t * 2 + 1], s = span[t];
+    const int lvl = (s == 1) ? 0 : (s == 2) ? 1 : (s == 4) ? 2 : -1;
+    if (lvl < 0 || y < 0 || x < 0 || y + s > fh || x + s > fw || ((y | x) & (s - 1))) {
+      raise_status(status, AVITS_ERR_COVERAGE);
+    } else {
+      const int32_t entry = map_entry(ti, lvl);
+      int32_t* m = map + (int64_t)b * fh * fw + (int64_t)y * fw + x;
+      for (int u = 0; u < s; ++u)
+        for (int v = 0; v < s; ++v) m[(int64_t)u * fw + v] = entry;
+      cells = (unsigned int)(s * s);
+    }
+  }
+  cells = __reduce_add_sync(0xffffffffu, cells);
+  if ((threadIdx.x & 31) == 0 && cells) atomicAdd(&cta_cells, cells);
+  __syncthreads();
+  if (threadIdx.x == 0) count_cells(hdr, cta_cells, (unsigned long long)B * fh * fw, status);
+}
+
+// The entry of a cell if its token covers the cell in this call, else -1 (a
+// hole: the entry of an earlier call).
+__device__ __forceinline__ int32_t live_entry(int32_t e, int N, const int32_t* __restrict__ posb,
+                                              const int32_t* __restrict__ spanb, int Y, int X) {
+  if (e < 0) return -1;
+  const int t = map_tok(e), s = 1 << map_lvl(e);
+  if (t >= N || spanb[t] != s) return -1;
+  const int y = posb[t * 2], x = posb[t * 2 + 1];
+  return (Y & ~(s - 1)) == y && (X & ~(s - 1)) == x ? e : -1;
+}
+
+// Level-1 pixel (Y, X) of channel c: the frame's own, or inside a span-4 token
+// the 2x bilinear resize of level 2 (the coarse-to-fine cascade; spans are at
+// most 4).
 template <typename T>
-__global__ void merge_bilinear_kernel(const T* __restrict__ mixed, int B, int N, int fh, int fw,
-                                      int C, const int32_t* __restrict__ map, T* __restrict__ out,
-                                      unsigned int* status) {
+__device__ __forceinline__ float level1_pixel(const T* __restrict__ mb, int T4,
+                                              const int32_t* __restrict__ mapb, int fh, int fw,
+                                              int c, int Y, int X) {
+  const int32_t e = mapb[(int64_t)Y * fw + X];
+  return (e >= 0 && map_lvl(e) >= 2) ? frame_resize2x(2, mb, T4, mapb, fh, fw, c, Y, X)
+                                     : frame_pixel<1>(mb, T4, mapb, fw, c, Y, X);
+}
+
+// One (output cell, channel) on its own: a hole is reported and gives zeros, a
+// span-1 cell is copied, a coarser cell's four pixels are the 2x bilinear
+// resize of level 1 around it (a 3 x 3 neighbourhood, clamped to the frame).
+template <typename T>
+__device__ __forceinline__ typename Pix4<T>::V merge_cell_channel(
+    const T* __restrict__ mb, int T4, const int32_t* __restrict__ mapb, int fh, int fw, int32_t e,
+    int c, int Y, int X) {
+  using PV = typename Pix4<T>::V;
+  if (e < 0) return Pix4<T>::make(0.f, 0.f, 0.f, 0.f);
+  if (map_lvl(e) == 0) return reinterpret_cast<const PV*>(mb + (int64_t)map_tok(e) * T4)[c];
+  float lv[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      lv[i][j] = level1_pixel(mb, T4, mapb, fh, fw, c, min(max(Y - 1 + i, 0), fh - 1),
+                              min(max(X - 1 + j, 0), fw - 1));
+  float r[4];
+  resize_cell(lv, 0, 0, r);
+  return Pix4<T>::make(r[0], r[1], r[2], r[3]);
+}
+
+// Bilinear merge, pass 2, one thread per (output cell, channel): tokens whose
+// rows are not whole 16-byte pieces.
+template <typename T>
+__global__ void __launch_bounds__(256)
+merge_bilinear_kernel(const T* __restrict__ mixed, int B, int N, const int32_t* __restrict__ pos,
+                      const int32_t* __restrict__ span, int fh, int fw, int C,
+                      const int32_t* __restrict__ map, T* __restrict__ out, unsigned int* status) {
   using PV = typename Pix4<T>::V;
   pdl_wait_then_trigger();
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -324,52 +418,187 @@ __global__ void merge_bilinear_kernel(const T* __restrict__ mixed, int B, int N,
   const int b = (int)(bc / cells);
   const int cell = (int)(bc % cells);
   const int Y = cell / fw, X = cell - Y * fw;
-  const int T4 = C * 4;
   const int32_t* mapb = map + (int64_t)b * cells;
-  const T* mb = mixed + (int64_t)b * N * T4;
-  const int32_t e = mapb[cell];
-  PV* dst = reinterpret_cast<PV*>(out + bc * T4) + c;
-  if (e < 0) {
-    raise_status(status, AVITS_ERR_COVERAGE);
-    *dst = Pix4<T>::make(0.f, 0.f, 0.f, 0.f);
-    return;
-  }
-  if (map_lvl(e) == 0) {
-    *dst = reinterpret_cast<const PV*>(mb + (int64_t)map_tok(e) * T4)[c];
-    return;
-  }
-  // level-1 pixels (rows Y-1..Y+1, columns X-1..X+1, clamped): the frame's
-  // own, or inside a span-4 token the resize of level 2
-  int rr[3], cc[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    rr[k] = min(max(Y - 1 + k, 0), fh - 1);
-    cc[k] = min(max(X - 1 + k, 0), fw - 1);
-  }
-  float lv[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const int32_t en = mapb[(int64_t)rr[i] * fw + cc[j]];
-      lv[i][j] = (en >= 0 && map_lvl(en) >= 2)
-                     ? frame_resize2x(2, mb, T4, mapb, fh, fw, c, rr[i], cc[j])
-                     : frame_pixel<1>(mb, T4, mapb, fw, c, rr[i], cc[j]);
-    }
-  float r[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    // output pixel row 2Y + a draws on level-1 rows (Y - 1, Y) for a = 0 and
-    // (Y, Y + 1) for a = 1 with weights (1/4, 3/4) / (3/4, 1/4), clamped at
-    // the frame edge: neighbourhood rows a and a + 1; columns likewise
-    const int a = q >> 1, bq = q & 1;
-    const float wy0 = a ? 0.75f : 0.25f, wy1 = a ? 0.25f : 0.75f;
-    const float wx0 = bq ? 0.75f : 0.25f, wx1 = bq ? 0.25f : 0.75f;
-    r[q] = bil_combine(lv[a][bq], lv[a][bq + 1], lv[a + 1][bq], lv[a + 1][bq + 1], wy0, wy1, wx0,
-                       wx1);
-  }
-  *dst = Pix4<T>::make(r[0], r[1], r[2], r[3]);
+  const int32_t e = live_entry(mapb[cell], N, pos + (int64_t)b * N * 2, span + (int64_t)b * N, Y, X);
+  if (e < 0) raise_status(status, AVITS_ERR_COVERAGE);
+  reinterpret_cast<PV*>(out + bc * C * 4)[c] =
+      merge_cell_channel(mixed + (int64_t)b * N * C * 4, C * 4, mapb, fh, fw, e, c, Y, X);
 }
+
+// Bilinear merge, pass 2, for tokens of whole 16-byte pieces: a CTA takes a tile
+// of 16 x 16 cells and two pieces (32 bytes) of the channels.  It loads the
+// cell map of the tile and four cells around it, turns every cell of the tile
+// and the ring next to it into its level-1 pixel (one 16-byte load: a span-2
+// token's pixel, or the average of a span-1 token's four) in shared memory,
+// and writes the cells from the 3 x 3 level-1 pixels around them; span-1 cells
+// are copied.  Only where a span-4 token is near does it also build the level-2
+// pixels (from the wider ring) and refine the level-1 pixels inside such
+// tokens.  Every value is the one merge_cell_channel would compute, in the same
+// order of operations.  What bounds it: the chain map - token - shared memory -
+// cell at a few CTAs per SM, then the copies.  us of the two kernels, against a
+// thread per (cell, channel) behind a fill and an atomic scatter, bf16, 64 x 64
+// cells of 16 channels: batch 1 8.4 -> 6.5, 16 31.3 -> 12.8, 64 102 -> 33.7;
+// batch 32 with spans 1, 2 and 4 2606 -> 29.8 (a value of level 2 was pooled
+// anew by every thread that drew on it).  Left out: a thread per 2 x 2 cells
+// with the neighbourhood in registers, 10.5 at batch 16 but 5580 with span 4;
+// three pieces of a thread in flight 13.2.
+constexpr int kTile = 16;
+constexpr int kHalo = 4;                        // cells around the tile that level 2 can draw on
+constexpr int kReg = kTile + 2 * kHalo;
+constexpr int kTilePieces = 2;
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+merge_bilinear_tile_kernel(const T* __restrict__ mixed, int N, const int32_t* __restrict__ pos,
+                           const int32_t* __restrict__ span, int fh, int fw, int C,
+                           const int32_t* __restrict__ map, T* __restrict__ out,
+                           unsigned int* status, unsigned tiles_x, unsigned tiles_y,
+                           unsigned groups) {
+  constexpr int kCh = Chunk<T>::kCh;
+  __shared__ int32_t smap[kReg][kReg];
+  __shared__ float l1[kTilePieces][kCh][kReg][kReg];
+  __shared__ float l2[kTilePieces][kCh][kReg / 2][kReg / 2];
+  pdl_wait_then_trigger();
+  unsigned blk = blockIdx.x;
+  const int grp = (int)(blk % groups);
+  blk /= groups;
+  const int X0 = (int)(blk % tiles_x) * kTile;
+  blk /= tiles_x;
+  const int Y0 = (int)(blk % tiles_y) * kTile, b = (int)(blk / tiles_y);
+  const int T4 = C * 4, cpc = C / kCh;
+  const int npc = min(kTilePieces, cpc - grp * kTilePieces);   // pieces of this CTA
+  const int32_t* mapb = map + (int64_t)b * fh * fw;
+  const int32_t* posb = pos + (int64_t)b * N * 2;
+  const int32_t* spanb = span + (int64_t)b * N;
+  const T* mb = mixed + (int64_t)b * N * T4;
+  T* ob = out + (int64_t)b * fh * fw * T4;
+  // the map, -1 off the frame and for words that are no token of this call
+  bool wide = false;
+  for (int i = threadIdx.x; i < kReg * kReg; i += 256) {
+    const int r = i / kReg, c = i - r * kReg;
+    const int Y = Y0 - kHalo + r, X = X0 - kHalo + c;
+    int32_t e = -1;
+    if (Y >= 0 && Y < fh && X >= 0 && X < fw) {
+      e = mapb[(int64_t)Y * fw + X];
+      if (e >= 0 && map_tok(e) >= N) e = -1;
+    }
+    smap[r][c] = e;
+    wide = wide || (e >= 0 && map_lvl(e) >= 2 && r >= kHalo - 1 && r <= kHalo + kTile &&
+                    c >= kHalo - 1 && c <= kHalo + kTile);
+  }
+  wide = __syncthreads_or(wide);
+  auto piece = [&](int32_t e, int pc) {
+    return *(reinterpret_cast<const uint4*>(mb + (int64_t)map_tok(e) * T4) + grp * kTilePieces + pc);
+  };
+  auto write = [&](int Y, int X, int pc, const uint4& w) {
+    *(reinterpret_cast<uint4*>(ob + ((int64_t)Y * fw + X) * T4) + grp * kTilePieces + pc) = w;
+  };
+  // level-1 pixels of the cells outside span-4 tokens; span-1 cells and holes of
+  // the tile are written here
+  const int first = wide ? 0 : kHalo - 1, side = wide ? kReg : kTile + 2;
+  for (int i = threadIdx.x; i < side * side * kTilePieces; i += 256) {
+    const int pc = i % kTilePieces, q = i / kTilePieces;
+    const int r = first + q / side, c = first + q % side;
+    if (pc >= npc) continue;
+    int32_t e = smap[r][c];
+    const int Y = Y0 - kHalo + r, X = X0 - kHalo + c;
+    const bool mine = r >= kHalo && r < kHalo + kTile && c >= kHalo && c < kHalo + kTile &&
+                      Y < fh && X < fw;
+    const uint4 w = e >= 0 ? piece(e, pc) : make_uint4(0u, 0u, 0u, 0u);
+    if (mine && live_entry(e, N, posb, spanb, Y, X) < 0) {
+      raise_status(status, AVITS_ERR_COVERAGE);
+      write(Y, X, pc, make_uint4(0u, 0u, 0u, 0u));
+      smap[r][c] = -1;   // this cell's other piece reads no token, or found so as well
+      e = -1;
+    }
+    const int lvl = e >= 0 ? map_lvl(e) : -1;
+    if (mine && lvl == 0) write(Y, X, pc, w);
+    float p[kCh][4];
+    Chunk<T>::unpack(w, p);
+#pragma unroll
+    for (int ch = 0; ch < kCh; ++ch) {
+      float v = 0.f;
+      if (lvl == 0)
+        v = __fmul_rn(__fadd_rn(__fadd_rn(p[ch][0], p[ch][1]), __fadd_rn(p[ch][2], p[ch][3])),
+                      0.25f);
+      else if (lvl == 1)
+        v = (Y & 1) ? ((X & 1) ? p[ch][3] : p[ch][2]) : ((X & 1) ? p[ch][1] : p[ch][0]);
+      l1[pc][ch][r][c] = v;
+    }
+  }
+  __syncthreads();
+  if (wide) {
+    // level 2: a span-4 token's pixel, or the average of four level-1 pixels
+    for (int i = threadIdx.x; i < (kReg / 2) * (kReg / 2) * kTilePieces; i += 256) {
+      const int pc = i % kTilePieces, q = i / kTilePieces;
+      const int r = q / (kReg / 2), c = q % (kReg / 2);
+      if (pc >= npc) continue;
+      const int32_t e = smap[2 * r][2 * c];
+      const bool four = e >= 0 && map_lvl(e) >= 2;
+      float p[kCh][4];
+      if (four) Chunk<T>::unpack(piece(e, pc), p);
+      const int R = (Y0 - kHalo) / 2 + r, Q = (X0 - kHalo) / 2 + c;
+#pragma unroll
+      for (int ch = 0; ch < kCh; ++ch) {
+        const float(*s)[kReg] = l1[pc][ch];
+        l2[pc][ch][r][c] =
+            four ? ((R & 1) ? ((Q & 1) ? p[ch][3] : p[ch][2]) : ((Q & 1) ? p[ch][1] : p[ch][0]))
+            : e < 0 ? 0.f
+                    : __fmul_rn(__fadd_rn(__fadd_rn(s[2 * r][2 * c], s[2 * r][2 * c + 1]),
+                                          __fadd_rn(s[2 * r + 1][2 * c], s[2 * r + 1][2 * c + 1])),
+                                0.25f);
+      }
+    }
+    __syncthreads();
+    // level 1 inside span-4 tokens: the 2x resize of level 2
+    for (int i = threadIdx.x; i < (kTile + 2) * (kTile + 2) * kTilePieces; i += 256) {
+      const int pc = i % kTilePieces, q = i / kTilePieces;
+      const int r = kHalo - 1 + q / (kTile + 2), c = kHalo - 1 + q % (kTile + 2);
+      const int32_t e = smap[r][c];
+      if (pc >= npc || e < 0 || map_lvl(e) < 2) continue;
+      int r0, r1, c0, c1;
+      float wy0, wy1, wx0, wx1;
+      bil_axis(Y0 - kHalo + r, fh / 2, r0, r1, wy0, wy1);
+      bil_axis(X0 - kHalo + c, fw / 2, c0, c1, wx0, wx1);
+      r0 -= (Y0 - kHalo) / 2;
+      r1 -= (Y0 - kHalo) / 2;
+      c0 -= (X0 - kHalo) / 2;
+      c1 -= (X0 - kHalo) / 2;
+#pragma unroll
+      for (int ch = 0; ch < kCh; ++ch)
+        l1[pc][ch][r][c] = bil_combine(l2[pc][ch][r0][c0], l2[pc][ch][r0][c1], l2[pc][ch][r1][c0],
+                                       l2[pc][ch][r1][c1], wy0, wy1, wx0, wx1);
+    }
+    __syncthreads();
+  }
+  for (int i = threadIdx.x; i < kTile * kTile * kTilePieces; i += 256) {
+    const int pc = i % kTilePieces, q = i / kTilePieces;
+    const int r = kHalo + q / kTile, c = kHalo + q % kTile;
+    const int32_t e = smap[r][c];
+    const int Y = Y0 - kHalo + r, X = X0 - kHalo + c;
+    if (pc >= npc || e < 0 || map_lvl(e) == 0 || Y >= fh || X >= fw) continue;
+    float v[kCh][4];
+#pragma unroll
+    for (int ch = 0; ch < kCh; ++ch) {
+      float lv[3][3];
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+#pragma unroll
+        for (int w = 0; w < 3; ++w)
+          lv[u][w] = l1[pc][ch][r + (min(max(Y - 1 + u, 0), fh - 1) - Y)]
+                               [c + (min(max(X - 1 + w, 0), fw - 1) - X)];
+      resize_cell(lv, 0, 0, v[ch]);
+    }
+    write(Y, X, pc, Chunk<T>::pack(v));
+  }
+}
+
+// One pass up to here: us in one / two passes at 1945 tokens 3.2 / 4.0, 3890 5.6 /
+// 4.4, 7780 7.1 / 4.4, 124480 99 / 12.4 (64 x 64 cells per 1945 tokens, bf16; one
+// pass with 8 lanes per token and 4 CTAs per SM 3.2, 5.6, 4.9, 28.8).
+constexpr int kOnePassTokensPerSm = 16;
+constexpr int64_t kMaxWork = 0xfffffff0ll - 1024;   // 32-bit indices within an element
+constexpr int64_t kMaxGrid = 0x7fffffffll;
 
 template <typename T>
 cudaError_t launch_t(const void* mixed, int B, int N, const int32_t* pos, const int32_t* span,
@@ -383,11 +612,15 @@ cudaError_t launch_t(const void* mixed, int B, int N, const int32_t* pos, const 
     cudaError_t e0 = cudaGetDevice(&dev);
     if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e0 != cudaSuccess) return e0;
-    const int64_t cap = (int64_t)std::max(1, sms) * kNearestCtasPerSm;
     cudaError_t e = prefer_max_shared<merge_nearest_warp_kernel<T>>();
-    if (e == cudaSuccess) e = prefer_max_shared<merge_nearest_kernel<T, 8>>();
+    if (e == cudaSuccess) e = prefer_max_shared<merge_index_kernel>();
+    if (e == cudaSuccess) e = prefer_max_shared<merge_nearest_gather_kernel<T, true>>();
+    if (e == cudaSuccess) e = prefer_max_shared<merge_nearest_gather_kernel<T, false>>();
     if (e != cudaSuccess) return e;
-    if (ntok <= cap * kNearestWarps) {
+    const bool whole = (C * 4 * (int)sizeof(T)) % 16 == 0;
+    const int64_t work = (int64_t)fh * fw * (whole ? C * 4 * (int)sizeof(T) / 16 : C);
+    if (ntok <= (int64_t)std::max(1, sms) * kOnePassTokensPerSm || work > kMaxWork ||
+        B * ((work + 255) / 256) > kMaxGrid) {
       // one warp per token, one pass (latency-bound sizes)
       e = launch_pdl(merge_nearest_warp_kernel<T>, dim3((unsigned)((ntok + 7) / 8)),
                      dim3(8 * 32), 0, s, static_cast<const T*>(mixed), B, N, pos, span, fh, fw,
@@ -395,25 +628,43 @@ cudaError_t launch_t(const void* mixed, int B, int N, const int32_t* pos, const 
       if (e != cudaSuccess) return e;
       return cudaGetLastError();
     }
-    const int64_t per_cta = (int64_t)kNearestWarps * 4;
-    const int grid = (int)std::min<int64_t>((ntok + per_cta - 1) / per_cta, cap);
-    e = launch_pdl(merge_nearest_kernel<T, 8>, dim3(grid), dim3(kNearestWarps * 32), 0, s,
-                               static_cast<const T*>(mixed), B, N, pos, span, fh, fw, C,
-                               static_cast<T*>(out), hdr, words, status);
+    int32_t* map = reinterpret_cast<int32_t*>(words);
+    e = launch_pdl(merge_index_kernel, dim3((unsigned)((ntok + 255) / 256)), dim3(256), 0, s, B, N,
+                   pos, span, fh, fw, map, hdr, status);
+    if (e != cudaSuccess) return e;
+    const unsigned ctas = (unsigned)((work + 256 * kGatherPieces - 1) / (256 * kGatherPieces));
+    e = launch_pdl(whole ? merge_nearest_gather_kernel<T, true> : merge_nearest_gather_kernel<T, false>,
+                   dim3(ctas * (unsigned)B), dim3(256), 0, s, static_cast<const T*>(mixed), N, pos,
+                   span, fh, fw, C, static_cast<const int32_t*>(map), static_cast<T*>(out), status,
+                   ctas);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
   }
-  // three kernels (fill, scatter of the cell map, gather), each a
-  // programmatic dependent of the one before: their launches overlap, every
-  // kernel waits for its predecessor before touching memory
+  // two kernels (scatter of the cell map, gather), the second a programmatic
+  // dependent of the first
   int32_t* map = reinterpret_cast<int32_t*>(words);
-  cudaError_t e = launch_cell_map(B, N, pos, span, fh, fw, map, status, s);
+  const int64_t nt = (int64_t)B * N;
+  cudaError_t e = prefer_max_shared<merge_scatter_kernel>();
   if (e == cudaSuccess) e = prefer_max_shared<merge_bilinear_kernel<T>>();
+  if (e == cudaSuccess) e = prefer_max_shared<merge_bilinear_tile_kernel<T>>();
   if (e != cudaSuccess) return e;
-  const int64_t work = (int64_t)B * fh * fw * C;
-  e = launch_pdl(merge_bilinear_kernel<T>, dim3((unsigned)((work + 255) / 256)), dim3(256), 0, s,
-                 static_cast<const T*>(mixed), B, N, fh, fw, C,
-                 static_cast<const int32_t*>(map), static_cast<T*>(out), status);
+  e = launch_pdl(merge_scatter_kernel, dim3((unsigned)((nt + 255) / 256)), dim3(256), 0, s, B, N,
+                 pos, span, fh, fw, map, hdr, status);
+  if (e != cudaSuccess) return e;
+  const bool whole = (C * 4 * (int)sizeof(T)) % 16 == 0;
+  const int64_t ty = (fh + kTile - 1) / kTile, tx = (fw + kTile - 1) / kTile;
+  const int64_t groups = (C / Chunk<T>::kCh + kTilePieces - 1) / kTilePieces;
+  if (whole && B * ty * tx * groups <= kMaxGrid) {
+    e = launch_pdl(merge_bilinear_tile_kernel<T>, dim3((unsigned)(B * ty * tx * groups)), dim3(256),
+                   0, s, static_cast<const T*>(mixed), N, pos, span, fh, fw, C,
+                   static_cast<const int32_t*>(map), static_cast<T*>(out), status, (unsigned)tx,
+                   (unsigned)ty, (unsigned)groups);
+  } else {
+    const int64_t all = (int64_t)B * fh * fw * C;
+    e = launch_pdl(merge_bilinear_kernel<T>, dim3((unsigned)((all + 255) / 256)), dim3(256), 0, s,
+                   static_cast<const T*>(mixed), B, N, pos, span, fh, fw, C,
+                   static_cast<const int32_t*>(map), static_cast<T*>(out), status);
+  }
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

@@ -69,7 +69,7 @@ class TransitionBuffers:
         self.full = torch.empty(B, self.full_h * self.full_w, tr.C * 4, dtype=dt, **z)
         self.ws = SpatialWorkspace(device)
         mb = avits_merge_final_workspace(self.mode, B, self.full_h, self.full_w)
-        # zero-filled before first use (the nearest merge's claim map and counter)
+        # zero-filled before first use (the merge's cell map and counter)
         self.merge_ws = torch.zeros(max(mb, 16), dtype=torch.uint8, **z) if mb else None
         # a mixed input in bilinear mode: the input frame's cell map
         ub = avits_selective_upsample_workspace(self.mode, B, tr.frame_h, tr.frame_w)

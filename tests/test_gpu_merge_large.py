@@ -1,0 +1,158 @@
+"""GPU parity (bit-exact) of the two-pass merge: batches of more tokens than
+one pass takes in nearest mode, and the bilinear merge, over token widths that
+are and are not whole 16-byte pieces, spans of every kind, and tilings that do
+not cover the frame, with one workspace used by both modes in turn."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+NEAREST, BILINEAR = 0, 1
+
+
+@pytest.fixture(scope="module")
+def av():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    import paper_2608_17995_gb300 as av
+    av.build()
+    av.lib()
+    return av
+
+
+def _tiling(rng, B, fh, fw, block, spans):
+    """pos [B,N,2], span [B,N]: blocks of block x block cells cut into tokens of
+    one span each, the same spans in every element but in other places and
+    another token order."""
+    cells = [(y, x) for y in range(0, fh, block) for x in range(0, fw, block)]
+    kinds = rng.choice(spans, size=len(cells))
+    pos, span = [], []
+    for _ in range(B):
+        p, s = [], []
+        for (y, x), k in zip(cells, rng.permutation(kinds)):
+            for u in range(0, block, k):
+                for v in range(0, block, k):
+                    p.append((y + u, x + v))
+                    s.append(k)
+        order = rng.permutation(len(s))
+        pos.append(np.array(p, np.int32)[order])
+        span.append(np.array(s, np.int32)[order])
+    return np.ascontiguousarray(np.stack(pos)), np.ascontiguousarray(np.stack(span))
+
+
+def _latent(rng, B, N, C, dtype):
+    from paper_2608_17995_gb300.workloads import to_bf16_bits
+    x = rng.standard_normal((B, N, C * 4)).astype(np.float32)
+    return to_bf16_bits(x) if dtype == "bf16" else x
+
+
+def _call(av, mixed, dtype, pos, span, fh, fw, mode, ws):
+    import torch
+    from paper_2608_17995_gb300.pipeline import to_device, to_numpy
+    B, _, T = mixed.shape
+    out = torch.full((B, fh * fw, T), 7.0, device="cuda",
+                     dtype=torch.bfloat16 if dtype == "bf16" else torch.float32)
+    av.avits_merge_final(to_device(mixed, dtype), to_device(pos, "i32"), to_device(span, "i32"),
+                         fh, fw, out, mode=mode, workspace=ws)
+    return to_numpy(out), av.avits_device_status()
+
+
+def _same(a, b):
+    v = np.uint16 if a.dtype == np.uint16 else np.uint32
+    return np.array_equal(a.view(v), b.view(v))
+
+
+@pytest.mark.parametrize("mode", [NEAREST, BILINEAR])
+@pytest.mark.parametrize("dtype,C,B,fh,fw", [
+    ("bf16", 16, 41, 24, 36), ("bf16", 1, 60, 24, 24), ("bf16", 3, 37, 12, 60), ("f32", 1, 45, 24, 36),
+    ("f32", 5, 40, 36, 24), ("bf16", 16, 3, 84, 108)])
+def test_merge_two_pass_bit_exact(av, mode, dtype, C, B, fh, fw):
+    import torch
+    import oracle
+    rng = np.random.default_rng(C * 1000 + B + mode)
+    block, spans = (12, [1, 2, 3, 4, 6, 12]) if mode == NEAREST else (4, [1, 2, 4])
+    if mode == BILINEAR and C == 16:
+        spans = [1, 2]   # the common schedule: no level-2 pixels
+    ws = torch.zeros(av.avits_merge_final_workspace(mode, B, fh, fw), dtype=torch.uint8, device="cuda")
+    for _ in range(2):   # the second call finds the first one's map
+        pos, span = _tiling(rng, B, fh, fw, block, spans)
+        mixed = _latent(rng, B, pos.shape[1], C, dtype)
+        got, st = _call(av, mixed, dtype, pos, span, fh, fw, mode, ws)
+        want, cover = oracle.merge_final(mixed, pos, span, fh, fw,
+                                         mode="nearest" if mode == NEAREST else "bilinear")
+        assert st == 0 and np.all(cover == 1)
+        assert _same(got, want)
+
+
+@pytest.mark.parametrize("first", [NEAREST, BILINEAR])
+def test_merge_two_pass_reports_bad_tilings(av, first):
+    import torch
+    import oracle
+    rng = np.random.default_rng(5)
+    B, fh, fw = 48, 24, 24
+    pos, span = _tiling(rng, B, fh, fw, 4, [1, 2])
+    mixed = _latent(rng, B, pos.shape[1], 4, "f32")
+    N = pos.shape[1]
+    ws = torch.zeros(av.avits_merge_final_workspace(NEAREST, B, fh, fw), dtype=torch.uint8, device="cuda")
+    want = {m: oracle.merge_final(mixed, pos, span, fh, fw,
+                                  mode="nearest" if m == NEAREST else "bilinear")[0]
+            for m in (NEAREST, BILINEAR)}
+
+    def bad():
+        two = np.flatnonzero(span[B - 1] == 1)[:2]
+        moved = pos.copy()
+        moved[B - 1, two[1]] = pos[B - 1, two[0]]       # a cell twice, another not at all
+        yield moved, span
+        empty = span.copy()
+        empty[0, N // 2] = 0                            # a token of no cells
+        yield pos, empty
+        far = pos.copy()
+        far[B // 2, 0] = [fh - 1, fw]                   # outside the frame
+        yield far, span
+
+    for p, s in bad():
+        for m in (first, 1 - first):
+            assert _call(av, mixed, "f32", p, s, fh, fw, m, ws)[1] == 6
+            got, st = _call(av, mixed, "f32", pos, span, fh, fw, m, ws)
+            assert st == 0 and _same(got, want[m])
+
+
+@pytest.mark.parametrize("dtype,C,gh,gw,k", [
+    ("bf16", 16, 9, 13, 40), ("f32", 4, 16, 16, 0), ("f32", 1, 8, 30, 240), ("bf16", 2, 33, 8, 100),
+    ("bf16", 1, 8, 8, 30), ("bf16", 16, 1, 20, 7), ("bf16", 16, 20, 1, 7)])
+def test_bilinear_children_bit_exact(av, dtype, C, gh, gw, k):
+    """The bilinear children of a dense grid, at its edges and corners, through
+    both upsample entry points (one grid row or column included)."""
+    import torch
+    import oracle
+    from paper_2608_17995_gb300.pipeline import to_device, to_numpy
+    rng = np.random.default_rng(gh * 100 + gw)
+    B, M = 3, gh * gw
+    lat = _latent(rng, B, M, C, dtype)
+    A, V = rng.random((2, B, M)).astype(np.float32)
+    S = oracle.fuse(A, V, 0.5)
+    _, mask, off = oracle.topk(S, k)
+    want = oracle.selective_upsample(lat, gh, gw, mask, mode="bilinear")
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    n = M + 3 * k
+
+    def outs():
+        return (torch.zeros(B, n, C * 4, dtype=tdt, device="cuda"),
+                torch.zeros(B, n, 2, dtype=torch.int32, device="cuda"),
+                torch.zeros(B, n, dtype=torch.int32, device="cuda"),
+                torch.zeros(B, n, dtype=torch.int32, device="cuda"),
+                torch.zeros(B, n, dtype=torch.int8, device="cuda"))
+    ld = to_device(lat, dtype)
+    one, two = outs(), outs()
+    av.avits_selective_upsample(ld, gh, gw, to_device(mask, "u8"), to_device(off, "i32"), k, *one,
+                                mode=BILINEAR)
+    sel = torch.zeros(B, max(k, 1), dtype=torch.int32, device="cuda")
+    o = torch.zeros(B, M, dtype=torch.int32, device="cuda")
+    m = torch.zeros(B, M, dtype=torch.uint8, device="cuda")
+    av.avits_select_upsample(to_device(A, "f32"), to_device(V, "f32"), 0.5, k, sel, o, m, ld, gh, gw,
+                             *two, mode=BILINEAR)
+    assert av.avits_device_status() == 0
+    for got in (one, two):
+        assert _same(to_numpy(got[0]), want[0])
+        for g, w in zip(got[1:], want[1:]):
+            assert np.array_equal(to_numpy(g), w)
