@@ -538,7 +538,7 @@ fuse_select_kernel(const SelArgs g) {
 // each warp upsamples its tokens from shared memory.  No CTA waits for
 // another.
 template <int kThreads, int kRegKeys, typename T, bool kBilinear>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 1)
 select_upsample_kernel(const SelArgs g, const UpsampleArgs<T> u, int parts, int stage_rows) {
   extern __shared__ uint32_t keys[];
   const int b = blockIdx.x / parts, part = blockIdx.x - b * parts;

@@ -11,10 +11,10 @@
 //                reading neighbouring pixels from the dense input latent, or,
 //                for a mixed input, from level log2(s) of the input frame's
 //                pixel pyramid through its cell map (frame_map.cuh).
-// Nearest with 16-byte token rows: each lane writes whole 16-byte chunks
-// (coalesced); otherwise lanes split the (child, channel) work, each writing
-// the 4 pixels of one channel of one child.  Lanes 0-3 write the position /
-// span / source maps.
+// Token rows of whole 16-byte chunks: each lane writes chunks (coalesced);
+// otherwise, and for the pixel pyramid of a mixed input, lanes split the
+// (child, channel) work, each writing the 4 pixels of one channel of one child.
+// Lanes 0-3 write the position / span / source maps.
 #pragma once
 
 #include "avits_common.cuh"
@@ -57,6 +57,62 @@ struct SharedRows {
   __device__ const T* row(int, int tok) const { return rows + (int64_t)(tok - lo) * T4; }
 };
 
+// 16-byte piece j of child (a, b) of the dense grid token (y, x), bilinear: its
+// 2 x 2 output pixels lie around the parent's pixel (a, b) and draw on the
+// 3 x 3 pixels around that one, which are in four tokens (own, and the
+// neighbours on the child's sides, clamped to the grid).  Rows and columns
+// are taken from the child's side: index 0 = towards the neighbour, 1 = the
+// parent's pixel, 2 = inside the own token; the weights are symmetric, so the
+// sums are those of the general path, term for term.
+template <typename T, typename Src>
+__device__ __forceinline__ uint4 bilinear_child(const Src& rows, int b_elem, int gh, int gw, int y,
+                                                int x, int a, int b, int j) {
+  constexpr int kCh = Chunk<T>::kCh;
+  const int yn = a ? min(y + 1, gh - 1) : max(y - 1, 0), xn = b ? min(x + 1, gw - 1) : max(x - 1, 0);
+  // the neighbour's pixel row / column next to the child: at the grid's edge
+  // the token is the own one and the pixel the parent's
+  const int pv = yn == y ? a : 1 - a, ph = xn == x ? b : 1 - b;
+  auto piece = [&](int ty, int tx, float (&p)[kCh][4]) {
+    Chunk<T>::unpack(*(reinterpret_cast<const uint4*>(rows.row(b_elem, ty * gw + tx)) + j), p);
+  };
+  float own[kCh][4], ver[kCh][4], hor[kCh][4], dia[kCh][4], out[kCh][4];
+  piece(y, x, own);
+  piece(yn, x, ver);
+  piece(y, xn, hor);
+  piece(yn, xn, dia);
+#pragma unroll
+  for (int c = 0; c < kCh; ++c) {
+    auto at = [&](const float (&p)[4], int r, int q) {
+      return r ? (q ? p[3] : p[2]) : (q ? p[1] : p[0]);
+    };
+    float g[3][3];
+    g[0][0] = at(dia[c], pv, ph);
+    g[0][1] = at(ver[c], pv, b);
+    g[0][2] = at(ver[c], pv, 1 - b);
+    g[1][0] = at(hor[c], a, ph);
+    g[2][0] = at(hor[c], 1 - a, ph);
+    g[1][1] = at(own[c], a, b);
+    g[1][2] = at(own[c], a, 1 - b);
+    g[2][1] = at(own[c], 1 - a, b);
+    g[2][2] = at(own[c], 1 - a, 1 - b);
+    // r[u][v]: u, v = 0 towards the neighbour, 1 inside
+    float r[2][2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int v = 0; v < 2; ++v)
+        r[u][v] = bil_combine(g[u][v], g[u][v + 1], g[u + 1][v], g[u + 1][v + 1], u ? 0.75f : 0.25f,
+                              u ? 0.25f : 0.75f, v ? 0.75f : 0.25f, v ? 0.25f : 0.75f);
+    const float t0 = a ? r[1][0] : r[0][0], t1 = a ? r[1][1] : r[0][1];
+    const float u0 = a ? r[0][0] : r[1][0], u1 = a ? r[0][1] : r[1][1];
+    out[c][0] = b ? t1 : t0;
+    out[c][1] = b ? t0 : t1;
+    out[c][2] = b ? u1 : u0;
+    out[c][3] = b ? u0 : u1;
+  }
+  return Chunk<T>::pack(out);
+}
+
 // Token i of element b, selected or not, starting at output o; one warp.
 // Src::row(b, tok) gives the token's source values (tok's bilinear
 // neighbours included).
@@ -87,10 +143,11 @@ __device__ __forceinline__ void upsample_token(const UpsampleArgs<T>& u, const S
   const T* src = rows.row(b, i);
   const int64_t out_tok0 = (int64_t)b * u.n_out + o;
   const int tb = T4 * (int)sizeof(T);
-  if (!kBilinear && (tb & 15) == 0) {
-    // 16-byte chunks: a deferred token is copied, a selected one gives each
-    // child (a, b) the chunk whose channel pixels all equal the parent's
-    // pixel (a, b); one chunk per lane (bf16, 16 channels: 32 lanes, 4 children)
+  if ((tb & 15) == 0 && (!kBilinear || !sel || !u.map)) {
+    // 16-byte chunks: a deferred token is copied; nearest gives each child
+    // (a, b) of a selected one the chunk whose channel pixels all equal the
+    // parent's pixel (a, b), bilinear on a dense grid resizes around it; one
+    // chunk per lane (bf16, 16 channels: 32 lanes, 4 children)
     const int cpc = tb / 16;
     if (!sel) {
       uint4* dst = reinterpret_cast<uint4*>(u.out + out_tok0 * T4);
@@ -99,8 +156,12 @@ __device__ __forceinline__ void upsample_token(const UpsampleArgs<T>& u, const S
       for (int q = lane; q < 4 * cpc; q += 32) {
         const int child = q / cpc, j = q - child * cpc;
         const int a = child >> 1, bb = child & 1;
-        reinterpret_cast<uint4*>(u.out + (out_tok0 + child) * T4)[j] =
-            gather_chunk<T>(src, j, a, a, bb, bb);
+        uint4 w;
+        if constexpr (kBilinear)
+          w = bilinear_child<T>(rows, b, gh, gw, y, x, a, bb, j);
+        else
+          w = gather_chunk<T>(src, j, a, a, bb, bb);
+        reinterpret_cast<uint4*>(u.out + (out_tok0 + child) * T4)[j] = w;
       }
     }
   } else if (!sel) {
