@@ -668,7 +668,8 @@ cudaError_t launch_fused_t(const SelArgs& g, const UpsampleArgs<T>& u, int B, in
       head + stage_rows * row_bytes > 96 * 1024)
     stage_rows = 0;
   const size_t smem = head + (size_t)stage_rows * row_bytes;
-  if (smem > 48 * 1024) {
+  // the 48 KB that need no opt-in hold the kernel's static arrays as well
+  if (smem > 40 * 1024) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
     if (e != cudaSuccess) return e;
   }
