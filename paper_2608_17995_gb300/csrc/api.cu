@@ -253,8 +253,9 @@ avits_status avits_score_spatiotemporal(const void* q_img, const void* k_all, av
     if (ws_bytes < spatial_tc_workspace(B, H, M, Nk, d, sms) || !workspace)
       return AVITS_ERR_INVALID_ARG;
     unsigned int* st = a.status;
+    const float beside_us = spatial_tc_estimate_us(B, H, M, Nk, d, sms);
     const LaunchHook temporal = [=](cudaStream_t ss) {
-      return launch_temporal_overlapped(h_t, h_prev, dt, B, M, D, eps, V, sms, st, ss);
+      return launch_temporal_overlapped(h_t, h_prev, dt, B, M, D, eps, V, sms, st, beside_us, ss);
     };
     return cuda_status(launch_spatial_tc(a, sms, s, &temporal));
   }

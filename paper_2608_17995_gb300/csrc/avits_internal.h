@@ -57,6 +57,8 @@ struct SpatialArgs {
 // layout is not eligible (the caller then uses the CUDA-core path).
 bool spatial_tc_eligible(const SpatialArgs& a);
 size_t spatial_tc_workspace(int B, int H, int M, int Nk, int d, int num_sms);
+// About how long the kernel takes at these sizes.
+float spatial_tc_estimate_us(int B, int H, int M, int Nk, int d, int num_sms);
 // Leading bytes of that workspace that must be zero before a call (the row
 // words and ready flags of the in-kernel merge); a completed call leaves them
 // zero again.
@@ -99,10 +101,11 @@ cudaError_t launch_wait_selftest(unsigned long long limit_ns, long long* result,
 cudaError_t launch_temporal(const void* ht, const void* hp, avits_dtype dt, int B, int N, int D,
                             float eps, float* V, int num_sms, unsigned int* status, cudaStream_t s);
 // The temporal score as a programmatic dependent of the kernel just launched
-// on `s`: one CTA per SM running beside it, waiting for it before exiting.
+// on `s`: CTAs running beside it, waiting for it before exiting.  beside_us:
+// about how long that kernel takes (only the split of the work depends on it).
 cudaError_t launch_temporal_overlapped(const void* ht, const void* hp, avits_dtype dt, int B,
                                        int N, int D, float eps, float* V, int num_sms,
-                                       unsigned int* status, cudaStream_t s);
+                                       unsigned int* status, float beside_us, cudaStream_t s);
 constexpr int kMaxSnapshots = 16;
 cudaError_t launch_temporal_var(const void* const* snaps, int n_t, avits_dtype dt, int B, int N,
                                 int D, float* V, int num_sms, cudaStream_t s);

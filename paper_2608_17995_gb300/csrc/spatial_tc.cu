@@ -817,6 +817,12 @@ size_t spatial_tc_workspace(int B, int H, int M, int Nk, int d, int num_sms) {
   return make_plan(B, H, M, Nk, num_sms).bytes;
 }
 
+float spatial_tc_estimate_us(int B, int H, int M, int Nk, int d, int num_sms) {
+  // ~6 us of start, merge and end, ~0.9 us per item of a CTA (d = 64: half the
+  // products, the same exponentials)
+  return 6.f + (d == 128 ? 0.9f : 0.75f) * (float)make_plan(B, H, M, Nk, num_sms).per;
+}
+
 size_t spatial_tc_zeroed_bytes(int B, int H, int M, int Nk, int d, int num_sms) {
   (void)d;
   return make_plan(B, H, M, Nk, num_sms).bytes;

@@ -19,6 +19,7 @@
 #include "avits_internal.h"
 
 #include <algorithm>
+#include <cmath>
 
 namespace avits {
 namespace {
@@ -139,8 +140,13 @@ temporal_scalar_kernel(const T* __restrict__ ht, const T* __restrict__ hp, int64
 
 // ------------------------------------------------ bulk-copy staged path --
 // 2 tokens (24 KB at D = 3072 bf16) per CTA-chunk: small enough to share an
-// SM with the spatial kernel's CTA, so the two can run concurrently.
+// SM with the spatial kernel's CTA, so the two can run concurrently.  Beside a
+// running kernel, where one CTA per SM has the work of all, narrower rows fill
+// the same 24 KB (a token per warp and more; D = 64: 19.7 -> 13.7 us for both
+// scores of 8 x 12 heads x 500 tokens).
 constexpr int kStageTokens = 2;
+constexpr int kOverlapBytes = 24 * 1024;
+constexpr int kOverlapMaxTokens = 64;
 constexpr int kStageBytesMax = 32 * 1024;
 
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -406,11 +412,14 @@ void launch_var_vec(const SnapPtrs& sp, int n_t, int64_t ntok, int D, float* V, 
 
 }  // namespace
 
+// beside_us (kOverlapped): about how long the running kernel takes.
 template <typename T, bool kOverlapped = false>
 cudaError_t launch_staged(const void* ht, const void* hp, int64_t ntok, int D, float eps, float* V,
-                          int num_sms, unsigned int* status, cudaStream_t s) {
+                          int num_sms, unsigned int* status, cudaStream_t s, float beside_us = 0.f) {
   const size_t row = (size_t)D * sizeof(T);
-  const int tpc = (int)std::min<size_t>(kStageTokens, kStageBytesMax / (2 * row));
+  int tpc = (int)std::min<size_t>(kStageTokens, kStageBytesMax / (2 * row));
+  if (kOverlapped)
+    tpc = std::max(tpc, (int)std::min<size_t>(kOverlapMaxTokens, kOverlapBytes / (2 * row)));
   const size_t smem = 2 * (size_t)tpc * row;
   static int done[64] = {};
   int dev = 0;
@@ -441,9 +450,22 @@ cudaError_t launch_staged(const void* ht, const void* hp, int64_t ntok, int D, f
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
   }
-  // one CTA per SM (it shares the SM with the running kernel's CTA)
+  // One CTA per SM shares the SM with the running kernel's CTA and reads about
+  // 10 KB per us (1.5 TB/s on 152 SMs); it cannot exit before that kernel has.
+  // When the running kernel ends before all is read, further CTAs take the
+  // rest at full speed, several to an SM and four chunks each.  Both scores,
+  // us one after the other / beside each other with one round / with this rule:
+  // 2048 tokens of 12 KB beside 16 us (8 x 24 heads x 256 queries) 22.1 / 24.3 / 22.6,
+  // 8192 beside 63 us 79.8 / 82 / 75.3, 2000 beside 11 us (4 heads) 17.7 / 20.8 / 16.2;
+  // with rounds by the bytes alone (two at 8192 tokens: one CTA per SM reads the
+  // second half) 96.4.  Where one round is enough further ones only delay the
+  // end: 4096 tokens beside 84 us 95.1 / 86.4, with two rounds 91.6.
+  const double meanwhile = 10.0e3 * std::max(num_sms, 1) * std::max(beside_us, 1.f);
+  const int64_t sms = std::max(num_sms, 1);
+  const bool enough = (double)ntok * 2.0 * (double)row <= meanwhile;
+  const int64_t rounds = enough ? 1 : std::max<int64_t>(2, (nchunks + 4 * sms - 1) / (4 * sms));
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)std::min<int64_t>(nchunks, (int64_t)std::max(num_sms, 1)));
+  cfg.gridDim = dim3((unsigned)std::min<int64_t>(nchunks, sms * std::min<int64_t>(rounds, 64)));
   cfg.blockDim = dim3(kWarpsPerCta * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -502,15 +524,15 @@ cudaError_t launch_temporal(const void* ht, const void* hp, avits_dtype dt, int 
 
 cudaError_t launch_temporal_overlapped(const void* ht, const void* hp, avits_dtype dt, int B,
                                        int N, int D, float eps, float* V, int num_sms,
-                                       unsigned int* status, cudaStream_t s) {
+                                       unsigned int* status, float beside_us, cudaStream_t s) {
   const int64_t ntok = (int64_t)B * N;
   const bool al = ((reinterpret_cast<uintptr_t>(ht) | reinterpret_cast<uintptr_t>(hp)) & 15u) == 0;
   const size_t row = (size_t)D * (dt == AVITS_BF16 ? 2 : 4);
   if (!(al && row % 16 == 0 && 2 * row <= (size_t)kStageBytesMax))
     return launch_temporal(ht, hp, dt, B, N, D, eps, V, num_sms, status, s);   // stream order
   return dt == AVITS_BF16
-             ? launch_staged<__nv_bfloat16, true>(ht, hp, ntok, D, eps, V, num_sms, status, s)
-             : launch_staged<float, true>(ht, hp, ntok, D, eps, V, num_sms, status, s);
+             ? launch_staged<__nv_bfloat16, true>(ht, hp, ntok, D, eps, V, num_sms, status, s, beside_us)
+             : launch_staged<float, true>(ht, hp, ntok, D, eps, V, num_sms, status, s, beside_us);
 }
 
 cudaError_t launch_temporal_var(const void* const* snaps, int n_t, avits_dtype dt, int B, int N,
