@@ -25,6 +25,7 @@ Calls:
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from typing import Optional, Sequence
 
@@ -128,9 +129,22 @@ def lib():
 
 
 # ------------------------------------------------------------- marshalling --
+# A call's host time is mostly here, so the helpers stay lean: a lookup of the
+# current stream as an object took 2.9 us (its raw handle 0.2), a size query
+# through ctypes 1.0, and an attention call 20.8 us in all, 4.5 of them in the
+# library.
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
+_Int64x3 = ctypes.c_int64 * 3
 
 
 def _ptr(t) -> Optional[int]:
@@ -144,8 +158,12 @@ def _ptr(t) -> Optional[int]:
 
 
 def _stream(stream) -> Optional[int]:
+    """The stream's handle; None: the current stream of the current device."""
     if stream is None:
-        return _torch().cuda.current_stream().cuda_stream
+        torch = _torch()
+        if not torch.cuda.is_initialized():
+            return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -192,6 +210,23 @@ def avits_score_spatial_workspace(dtype, B, H, M, Nk, d) -> int:
     return int(lib().avits_score_spatial_workspace(code, B, H, M, Nk, d))
 
 
+@functools.lru_cache(maxsize=256)
+def _spatial_need(device: int, code: int, B: int, H: int, M: int, Nk: int, d: int) -> int:
+    """The same by sizes and device (the query depends on nothing else)."""
+    return int(lib().avits_score_spatial_workspace(code, B, H, M, Nk, d))
+
+
+def _spatial_ws(code, q_img, B, H, M, Nk, d, workspace, stream):
+    """Buffer and bytes for a spatial score on the current device."""
+    need = _spatial_need(_torch().cuda.current_device(), code, B, H, M, Nk, d)
+    if workspace is None:
+        key = (q_img.device.index, stream)
+        workspace = _default_ws.get(key)
+        if workspace is None:
+            workspace = _default_ws.setdefault(key, SpatialWorkspace(q_img.device))
+    return workspace.get(need)
+
+
 class SpatialWorkspace:
     """Device scratch for avits_score_spatial, grown on demand (reused by
     calls on one stream).  Allocated zero-filled: the counters at its start
@@ -230,34 +265,28 @@ def avits_score_spatial(q_img, k_all, L: int, softmax_scale: float, A, weight: f
     Nk = k_all.shape[2]
     if k_all.shape[0] != B or k_all.shape[1] != H or k_all.shape[3] != d:
         raise ValueError("q_img / k_all shapes disagree")
-    if q_img.stride(3) != 1 or k_all.stride(3) != 1:
+    qs, ks = q_img.stride(), k_all.stride()
+    if qs[3] != 1 or ks[3] != 1:
         raise ValueError("the head-dim axis must be contiguous")
     dt = _dtype_code(q_img)
     if _dtype_code(k_all) != dt:
         raise TypeError("q_img and k_all dtypes differ")
-    need = int(lib().avits_score_spatial_workspace(dt, B, H, M, Nk, d))
-    if workspace is None:
-        key = (q_img.device.index, _torch().cuda.current_stream().cuda_stream if stream is None else _stream(stream))
-        workspace = _default_ws.setdefault(key, SpatialWorkspace(q_img.device))
-    wbuf, wbytes = workspace.get(need)
+    stream = _stream(stream)
+    wbuf, wbytes = _spatial_ws(dt, q_img, B, H, M, Nk, d, workspace, stream)
     if text_mask is not None:
         if tuple(text_mask.shape) != (B, Nk) or text_mask.element_size() != 1 or \
                 not text_mask.is_contiguous():
             raise ValueError("text_mask must be a contiguous [B,Nk] byte tensor")
         rc = lib().avits_score_spatial_keymask(
-            _ptr(q_img), _ptr(k_all), dt, B, H, M, Nk, d,
-            q_img.stride(0), q_img.stride(1), q_img.stride(2),
-            k_all.stride(0), k_all.stride(1), k_all.stride(2), _ptr(text_mask),
-            float(softmax_scale), float(weight), 1 if accumulate else 0,
-            _ptr(A), _ptr(lse), _ptr(wbuf), wbytes, _stream(stream))
+            _ptr(q_img), _ptr(k_all), dt, B, H, M, Nk, d, qs[0], qs[1], qs[2], ks[0], ks[1],
+            ks[2], _ptr(text_mask), float(softmax_scale), float(weight), 1 if accumulate else 0,
+            _ptr(A), _ptr(lse), _ptr(wbuf), wbytes, stream)
         _check("avits_score_spatial_keymask", rc)
         return A
     rc = lib().avits_score_spatial(
-        _ptr(q_img), _ptr(k_all), dt, B, H, M, Nk, L, d,
-        q_img.stride(0), q_img.stride(1), q_img.stride(2),
-        k_all.stride(0), k_all.stride(1), k_all.stride(2),
+        _ptr(q_img), _ptr(k_all), dt, B, H, M, Nk, L, d, qs[0], qs[1], qs[2], ks[0], ks[1], ks[2],
         float(softmax_scale), float(weight), 1 if accumulate else 0,
-        _ptr(A), _ptr(lse), _ptr(wbuf), wbytes, _stream(stream))
+        _ptr(A), _ptr(lse), _ptr(wbuf), wbytes, stream)
     _check("avits_score_spatial", rc)
     return A
 
@@ -273,24 +302,20 @@ def avits_score_spatial_lse(q_img, k_txt, lse_all, softmax_scale: float, A, weig
     L = k_txt.shape[2]
     if k_txt.shape[0] != B or k_txt.shape[1] != H or k_txt.shape[3] != d:
         raise ValueError("q_img / k_txt shapes disagree")
-    if q_img.stride(3) != 1 or k_txt.stride(3) != 1:
+    qs, ks = q_img.stride(), k_txt.stride()
+    if qs[3] != 1 or ks[3] != 1:
         raise ValueError("the head-dim axis must be contiguous")
     if tuple(lse_all.shape) != (B, H, M) or not lse_all.is_contiguous():
         raise ValueError("lse_all must be a contiguous [B,H,M] tensor")
     dt = _dtype_code(q_img)
     if _dtype_code(k_txt) != dt:
         raise TypeError("q_img and k_txt dtypes differ")
-    need = int(lib().avits_score_spatial_workspace(dt, B, H, M, L, d))
-    if workspace is None:
-        key = (q_img.device.index, _torch().cuda.current_stream().cuda_stream if stream is None else _stream(stream))
-        workspace = _default_ws.setdefault(key, SpatialWorkspace(q_img.device))
-    wbuf, wbytes = workspace.get(need)
+    stream = _stream(stream)
+    wbuf, wbytes = _spatial_ws(dt, q_img, B, H, M, L, d, workspace, stream)
     rc = lib().avits_score_spatial_lse(
-        _ptr(q_img), _ptr(k_txt), dt, B, H, M, L, d,
-        q_img.stride(0), q_img.stride(1), q_img.stride(2),
-        k_txt.stride(0), k_txt.stride(1), k_txt.stride(2), _ptr(lse_all),
-        float(softmax_scale), float(weight), 1 if accumulate else 0,
-        _ptr(A), _ptr(lse), _ptr(wbuf), wbytes, _stream(stream))
+        _ptr(q_img), _ptr(k_txt), dt, B, H, M, L, d, qs[0], qs[1], qs[2], ks[0], ks[1], ks[2],
+        _ptr(lse_all), float(softmax_scale), float(weight), 1 if accumulate else 0,
+        _ptr(A), _ptr(lse), _ptr(wbuf), wbytes, stream)
     _check("avits_score_spatial_lse", rc)
     return A
 
@@ -304,23 +329,19 @@ def avits_score_spatiotemporal(q_img, k_all, L: int, softmax_scale: float, A, h_
     B, H, M, d = q_img.shape
     Nk = k_all.shape[2]
     D = h_t.shape[2]
-    if q_img.stride(3) != 1 or k_all.stride(3) != 1:
+    qs, ks = q_img.stride(), k_all.stride()
+    if qs[3] != 1 or ks[3] != 1:
         raise ValueError("the head-dim axis must be contiguous")
     if not (h_t.is_contiguous() and h_prev.is_contiguous()) or tuple(h_t.shape[:2]) != (B, M):
         raise ValueError("h_t / h_prev must be contiguous [B, M, D]")
     dt = _dtype_code(q_img)
-    need = int(lib().avits_score_spatial_workspace(dt, B, H, M, Nk, d))
-    if workspace is None:
-        key = (q_img.device.index, _stream(stream))
-        workspace = _default_ws.setdefault(key, SpatialWorkspace(q_img.device))
-    wbuf, wbytes = workspace.get(need)
+    stream = _stream(stream)
+    wbuf, wbytes = _spatial_ws(dt, q_img, B, H, M, Nk, d, workspace, stream)
     rc = lib().avits_score_spatiotemporal(
-        _ptr(q_img), _ptr(k_all), dt, B, H, M, Nk, L, d,
-        q_img.stride(0), q_img.stride(1), q_img.stride(2),
-        k_all.stride(0), k_all.stride(1), k_all.stride(2),
+        _ptr(q_img), _ptr(k_all), dt, B, H, M, Nk, L, d, qs[0], qs[1], qs[2], ks[0], ks[1], ks[2],
         float(softmax_scale), float(weight), 1 if accumulate else 0,
         _ptr(A), _ptr(lse), _ptr(wbuf), wbytes, _ptr(h_t), _ptr(h_prev), D, float(eps), _ptr(V),
-        _stream(stream))
+        stream)
     _check("avits_score_spatiotemporal", rc)
     return A, V
 
@@ -329,9 +350,9 @@ def avits_attention_forward_workspace(B: int, H: int, Mq: int) -> int:
     return int(lib().avits_attention_forward_workspace(B, H, Mq))
 
 
-def _strides3(t):
-    arr = (ctypes.c_int64 * 3)(t.stride(0), t.stride(1), t.stride(2))
-    return arr
+@functools.lru_cache(maxsize=256)
+def _attention_need(B: int, H: int, Mq: int) -> int:
+    return avits_attention_forward_workspace(B, H, Mq)
 
 
 def avits_attention_forward(q, k, v, L: int, softmax_scale: float, o, lse=None, A=None,
@@ -347,25 +368,25 @@ def avits_attention_forward(q, k, v, L: int, softmax_scale: float, o, lse=None, 
     if tuple(k.shape) != (B, H, Nk, d) or tuple(v.shape) != (B, H, Nk, d) or \
             tuple(o.shape) != (B, H, Mq, d):
         raise ValueError("q / k / v / o shapes disagree")
-    for t in (q, k, v, o):
-        if t.stride(3) != 1:
+    strides = (q.stride(), k.stride(), v.stride(), o.stride())
+    for t in strides:
+        if t[3] != 1:
             raise ValueError("the head-dim axis must be contiguous")
     dt = _dtype_code(q)
     if _dtype_code(k) != dt or _dtype_code(v) != dt or _dtype_code(o) != dt:
         raise TypeError("q, k, v and o dtypes differ")
     wbuf, wbytes = None, 0
+    stream = _stream(stream)
     if A is not None:
-        need = avits_attention_forward_workspace(B, H, Mq)
         if workspace is None:
-            key = ("attn", q.device.index,
-                   _torch().cuda.current_stream().cuda_stream if stream is None else _stream(stream))
+            key = ("attn", q.device.index, stream)
             workspace = _default_ws.setdefault(key, SpatialWorkspace(q.device))
-        wbuf, wbytes = workspace.get(need)
-    qs, ks, vs, os_ = _strides3(q), _strides3(k), _strides3(v), _strides3(o)
+        wbuf, wbytes = workspace.get(_attention_need(B, H, Mq))
+    qs, ks, vs, os_ = (_Int64x3(t[0], t[1], t[2]) for t in strides)
     rc = lib().avits_attention_forward(
         _ptr(q), _ptr(k), _ptr(v), dt, B, H, Mq, Nk, L, d, qs, ks, vs, os_,
         float(softmax_scale), _ptr(o), _ptr(lse), float(weight), 1 if accumulate else 0,
-        _ptr(A), _ptr(wbuf), wbytes, _stream(stream))
+        _ptr(A), _ptr(wbuf), wbytes, stream)
     _check("avits_attention_forward", rc)
     return o
 

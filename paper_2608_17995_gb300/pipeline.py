@@ -9,7 +9,7 @@ from __future__ import annotations
 
 import numpy as np
 
-from . import (BILINEAR, NEAREST, SpatialWorkspace, avits_fuse_select, avits_merge_final,
+from . import (BILINEAR, NEAREST, SpatialWorkspace, _stream, avits_fuse_select, avits_merge_final,
                avits_merge_final_workspace, avits_score_spatial, avits_score_spatiotemporal,
                avits_score_temporal, avits_select_upsample, avits_selective_upsample,
                avits_selective_upsample_workspace)
@@ -120,8 +120,7 @@ class TransitionBuffers:
         kernel overlapping the spatial one, unless fused_scores=False), then
         selection and selective upsampling (one launch unless
         fused_tail=False) and the final merge."""
-        import torch
-        main = stream if stream is not None else torch.cuda.current_stream()
+        main = _stream(stream)   # looked up once for all the calls
         if fused_scores:
             self.scores(main)
         else:
