@@ -15,41 +15,59 @@
 // runs over all key tiles (128 keys), so O and the row statistics stay in
 // the CTA and no partial results cross CTAs (except Eq. 3's head sum).
 //
-// Tensor memory (512 columns): one S buffer of 128 columns that the two query
-// tiles take in turn (S_0(g), S_1(g), S_0(g+1), ...), P_t as bf16 pairs (64
-// columns per tile), O_t (D columns per tile).  S is free as soon as its
-// softmax has loaded it, so the other tile's S runs on the tensor pipe while
-// this one's exponentials are computed; P never goes through shared memory
-// (the PV product reads it from tensor memory), which leaves shared memory
-// for Q, a 4-stage K / V ring and the O staging: per key tile and SM the
-// operand reads are 128 KB (S) + 64 KB (V), the copies 64 KB.
+// Tensor memory (512 columns): S_t (128 columns per query tile), whose first
+// 64 columns are overwritten by P_t (bf16 pairs) as the softmax goes, and O_t
+// (D columns per tile).  S_t(g+1) is issued right behind the PV product that
+// reads P_t(g), by the same thread, so the two never overlap; while one tile's
+// softmax runs, the tensor pipe works on the other tile's PV and S.
 //
 // Roles (12 warps):
 //   warp 0       TMA producer: Q tiles, then the K and V tiles through a
-//                4-stage ring in the order the MMAs consume them (K_0, K_1,
-//                V_0, K_2, V_1, ...), 128-byte swizzle; a stage is refilled
-//                two key tiles after its last use.
+//                4-stage ring (8 at d = 64) in the order the MMAs consume them
+//                (K_0, V_0, K_1, V_1, ...), 128-byte swizzle.
 //   warps 1, 2   MMA issuers of query tile 0 / 1 (warp 1 owns tensor
-//                memory): for key tile g, S_t(g) = Q_t K_g^T (from shared
-//                memory) once the S before it has been loaded, then O_t +=
-//                P_t(g-1) V_(g-1) (A = P_t from tensor memory, the
-//                tcgen05.mma TS form; V read in its natural [keys, d] layout
-//                as an MN-major shared-memory operand, no transpose copy) once
-//                that P has been written.
+//                memory), in turns: O_t += P_t(g) V_g (A = P_t from tensor
+//                memory, the tcgen05.mma TS form; V read in its natural
+//                [keys, d] layout as an MN-major shared-memory operand, no
+//                transpose copy) in two 64-key halves, each as soon as its
+//                half of P is written, then S_t(g+1) = Q_t K_(g+1)^T.  The
+//                turns keep the tiles half a period apart: without them both
+//                softmaxes ran at the same time, shared the MUFU, and then
+//                both waited for the pipe (4570 clocks per key tile).  A warp
+//                waits for its operands during the other's turn: a wait costs
+//                it ~190 clocks even when the barrier has completed, and one
+//                warp issuing for both tiles spent 3600 clocks per key tile
+//                on six of them.
 //   warp 3       no role.
 //   warps 4-7    softmax and epilogue of query tile 0, warps 8-11 of tile 1:
-//                one row per thread (TMEM lane); the row's 128 S columns are
-//                loaded into registers and the S buffer released; the row
-//                maximum; the running maximum is raised only when a key
-//                tile's maximum exceeds it by more than 2^8 (P <= 256
-//                otherwise, no loss in bf16 or the fp32 accumulator), and then
-//                l and O are rescaled (O in tensor memory, by the whole warp);
-//                the exponentials (packed FMA + MUFU), the fp32 sums over all
-//                keys and over the text keys (the only addition the score
-//                needs) and the bf16 P row, written to tensor memory once the
-//                previous PV product has read P_t.  The epilogue divides O by
-//                the row sum and stores it 64 columns at a time through a
-//                swizzled staging block with a bulk tensor copy.
+//                one row per thread (TMEM lane), 64 keys at a time:
+//                exponentials against the running reference m (packed FMA +
+//                MUFU), the fp32 sums over all keys and over the text keys
+//                (the only addition the score needs), the bf16 P half to
+//                tensor memory.  The row maximum is not taken on this path
+//                (it cost 480 of a tile's 2300 clocks): m is the maximum of
+//                the row's first key tile and moves, to a half's maximum, only
+//                when that half's sum reaches 2^16 (or is NaN); l and O are
+//                then rescaled.  The epilogue divides O by the row sum and
+//                stores it 64 columns at a time through a swizzled staging
+//                block with a bulk tensor copy.  These warps take 208
+//                registers, the others 88 (at 168 each the compiler spilled).
+//
+// What bounds it: the chain of one tile's step, S product and its completion
+// (~900 clocks; 8 products whose operands leave shared memory at its 128 bytes
+// a clock), two halves of load, exponentials and store (~1600), waits (~200),
+// the second half's PV product; the pipe itself needs ~2290 clocks per key tile
+// for both tiles.  24 heads of 128, one image at 1024^2 (1536 x 1536): 27.2 ->
+// 25.9 us; at 2048^2 (4608 x 4608): 197 -> 177 us (1478 TFLOP/s, 0.78 of the
+// measured bf16 peak); batch 2: 395 -> 348 us, 413 -> 373 where logits rise along
+// the keys.  Without the care for P's rounding (kBig) 23.8 / 164 / 327 us, but the
+// error of O against 64 bits was then 3 to 6 % above the earlier kernel's; with
+// it 1 to 2 % below (kBig 2^8: equal, 2^6: 5 % below, 355 us).  References moved
+// from 2^9 on instead: equal, 370 us.
+// Measured and left out at 2048^2 (against 164): 16 softmax warps, two threads
+// per row (186 us); S in 64-key products with the next step's S behind this
+// step's PV (186: half-width products read Q twice); the turn passed before the
+// S product is issued (192); a jumped row's redo as a loop around the half (228).
 // Every wait is bounded (avits_common.cuh); after a timeout every role skips
 // its remaining work, drains what it issued and the CTA releases tensor
 // memory and exits.
@@ -70,7 +88,9 @@ constexpr int kQTiles = 2;          // query tiles per unit
 constexpr int kUnitRows = kBM * kQTiles;
 constexpr int kThreads = 12 * 32;
 constexpr int kTmemCols = 512;
-constexpr float kTau = 8.f;         // lazy rescale threshold (log2 units)
+constexpr int kHalf = kBN / 2;      // keys the softmax handles at a time
+constexpr float kJump = 0x1p16f;    // a half's sum from which the reference moves
+constexpr float kBig = 0x1p7f;      // and from which P's rounding is made up for
 constexpr uint32_t kIdescS = idesc_bf16(kBM, kBN, false);
 
 template <int D>
@@ -87,15 +107,14 @@ struct Cfg {
 constexpr int kStageTileBytes = kBM * 128;
 constexpr int kStageBytes = kQTiles * kStageTileBytes;
 constexpr int kMaxStages = 8;
-// Tensor memory columns: the S buffer both query tiles share, then P_t (bf16
-// pairs, 64 columns per tile), then O_t (D columns per tile).
-constexpr int kColS = 0, kColP = kBN, kColO = kBN + kQTiles * (kBN / 2);
+// Tensor memory columns: S_t (P_t in the first half of its columns), then O_t.
+constexpr int kColS = 0, kColO = kQTiles * kBN;
 
 struct Bars {
   uint64_t q_full[kQTiles], q_empty[kQTiles];
   uint64_t kv_full[kMaxStages], kv_empty[kMaxStages];
-  uint64_t s_full[kQTiles], s_empty[kQTiles], p_full[kQTiles], pv_done[kQTiles];
-  uint64_t o_full[kQTiles], o_empty[kQTiles], drain[kQTiles];
+  uint64_t s_full[kQTiles], p_full[kQTiles][2], pv_half[kQTiles];
+  uint64_t o_full[kQTiles], o_empty[kQTiles], turn[kQTiles], drain[kQTiles];
   uint32_t tmem_base;
   int abort;
 };
@@ -131,107 +150,150 @@ __device__ __forceinline__ bool bar_and(int id, int count, bool v) {
   return r != 0;
 }
 
-// Row maximum of 32 S columns whose first key is col0; keys >= Nk are left
-// out (kFull: all 32 are valid).
-template <bool kFull>
-__device__ __forceinline__ float chunk_max(const uint32_t (&r)[32], int col0, int Nk) {
-  float v[32];
+// Row maximum of 64 S columns whose first key is key0; with kGeneral keys >= Nk
+// are left out.
+template <bool kGeneral>
+__device__ __forceinline__ float half_max(const uint32_t (&a)[32], const uint32_t (&b)[32],
+                                          int key0, int Nk) {
+  float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-  for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
-  if (!kFull) {
-#pragma unroll
-    for (int e = 0; e < 32; ++e)
-      if (col0 + e >= Nk) v[e] = -INFINITY;
+  for (int e = 0; e < 32; ++e) {
+    float x = __uint_as_float(a[e]), y = __uint_as_float(b[e]);
+    if (kGeneral && key0 + e >= Nk) x = -INFINITY;
+    if (kGeneral && key0 + 32 + e >= Nk) y = -INFINITY;
+    m[e & 3] = max3(m[e & 3], x, y);
   }
-  float t[11];
-#pragma unroll
-  for (int g = 0; g < 10; ++g) t[g] = max3(v[3 * g], v[3 * g + 1], v[3 * g + 2]);
-  t[10] = fmaxf(v[30], v[31]);
-  const float u0 = max3(t[0], t[1], t[2]), u1 = max3(t[3], t[4], t[5]);
-  const float u2 = max3(t[6], t[7], t[8]);
-  return fmaxf(max3(u0, u1, u2), fmaxf(t[9], t[10]));
+  return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
 }
 
-// O_t row *= f (D fp32 columns at tO), 16 columns at a time.
+// O_t row *= f (D fp32 columns at tO), 64 columns at a time.
 template <int D>
 __device__ __forceinline__ void rescale_o(uint32_t tO, float f) {
 #pragma unroll 1
-  for (int k = 0; k < D / 16; ++k) {
-    uint32_t r[16];
-    tmem_ld16(tO + 16 * k, r);
-    tmem_wait(r);
+  for (int k = 0; k < D; k += 64) {
+    uint32_t a[32], b[32];
+    tmem_ld64_wait(tO + (uint32_t)k, a, b);
 #pragma unroll
-    for (int e = 0; e < 16; e += 2) {
-      float a0 = __uint_as_float(r[e]), a1 = __uint_as_float(r[e + 1]);
-      fmul2(a0, a1, f);
-      r[e] = __float_as_uint(a0);
-      r[e + 1] = __float_as_uint(a1);
+    for (int e = 0; e < 32; ++e) {
+      a[e] = __float_as_uint(__uint_as_float(a[e]) * f);
+      b[e] = __float_as_uint(__uint_as_float(b[e]) * f);
     }
-    tmem_st16(tO + 16 * k, r);
+    tmem_st32(tO + (uint32_t)k, a);
+    tmem_st32(tO + (uint32_t)k + 32, b);
   }
 }
 
-// Exponentials of 32 S columns (first key col0) against the running maximum
-// m, their fp32 sums over all keys and over the text keys, and the bf16
-// numerators packed in place: r[i] (i < 16) = keys 2i, 2i + 1 (the even key in
-// the low half), the layout the PV product reads P_t in from tensor memory.
-// kKind: 0 = valid image keys, 1 = valid text keys, 2 = general (keys beyond
-// Nk give 0, text keys counted one by one).
-template <int kKind>
-__device__ __forceinline__ void exp_chunk(uint32_t (&r)[32], int col0, int Nk, int L, float c,
-                                          float m, float& la, float& lt) {
+// Exponentials of 64 S columns (a: the first 32, b: the next; first key key0)
+// against the reference m, their fp32 sum, the sum over the text keys, and the
+// bf16 numerators: w[i] = keys 2i, 2i + 1 (the even key in the low half), the
+// layout the PV product reads P_t in from tensor memory.  kGeneral: keys
+// beyond Nk give 0 and text keys are counted one by one (else all 64 keys are
+// valid, and text keys or not).
+template <bool kGeneral>
+__device__ __forceinline__ void exp_half(const uint32_t (&a)[32], const uint32_t (&b)[32],
+                                         uint32_t (&w)[32], int key0, int Nk, int L, float c,
+                                         float m, float& sum, float& text) {
   const float nm = -m;
-  float s0 = 0.f, s1 = 0.f, t0 = 0.f;
+  float s[4] = {0.f, 0.f, 0.f, 0.f}, t = 0.f;
 #pragma unroll
-  for (int e = 0; e < 32; e += 2) {
+  for (int e = 0; e < 64; e += 2) {
+    const uint32_t r0 = e < 32 ? a[e & 31] : b[e & 31], r1 = e < 32 ? a[(e & 31) + 1] : b[(e & 31) + 1];
     float x0, x1;
-    ffma2(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), c, nm, x0, x1);
+    ffma2(__uint_as_float(r0), __uint_as_float(r1), c, nm, x0, x1);
     float e0 = ex2(x0), e1 = ex2(x1);
-    if (kKind == 2) {
-      if (col0 + e >= Nk) e0 = 0.f;
-      if (col0 + e + 1 >= Nk) e1 = 0.f;
-      if (col0 + e < L) t0 += e0;
-      if (col0 + e + 1 < L) t0 += e1;
+    if (kGeneral) {
+      if (key0 + e >= Nk) e0 = 0.f;
+      if (key0 + e + 1 >= Nk) e1 = 0.f;
+      if (key0 + e < L) t += e0;
+      if (key0 + e + 1 < L) t += e1;
     }
-    fadd2(s0, s1, e0, e1);
-    r[e >> 1] = pack_bf16x2(e0, e1);   // slot e / 2 <= e has been read
+    fadd2(s[(e & 2)], s[(e & 2) + 1], e0, e1);
+    w[e >> 1] = pack_bf16x2(e0, e1);
   }
-  const float cs = s0 + s1;
-  la += cs;
-  if (kKind == 1) lt += cs;
-  if (kKind == 2) lt += t0;
+  sum = (s[0] + s[1]) + (s[2] + s[3]);
+  text = kGeneral ? t : key0 < L ? sum : 0.f;
 }
 
-template <int kKind>
-__device__ __forceinline__ void exp_tile(uint32_t (&r0)[32], uint32_t (&r1)[32],
-                                         uint32_t (&r2)[32], uint32_t (&r3)[32], int key0,
-                                         int Nk, int L, float c, float m, float& la, float& lt) {
-  exp_chunk<kKind>(r0, key0, Nk, L, c, m, la, lt);
-  exp_chunk<kKind>(r1, key0 + 32, Nk, L, c, m, la, lt);
-  exp_chunk<kKind>(r2, key0 + 64, Nk, L, c, m, la, lt);
-  exp_chunk<kKind>(r3, key0 + 96, Nk, L, c, m, la, lt);
-}
-
-// The 16 packed words at the front of r (32 keys of P) into 16 tensor-memory
-// columns of this thread's lane.
-__device__ __forceinline__ void tmem_st_p(uint32_t taddr, const uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-      "%11, %12, %13, %14, %15, %16};" ::"r"(taddr),
-      AVITS_I8(0), AVITS_I8(8)
-      : "memory");
+// The sum of the bf16 numerators of a half.
+__device__ __forceinline__ float rounded_sum(const uint32_t (&w)[32]) {
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int e = 0; e < 32; ++e)
+    fadd2(s[2 * (e & 1)], s[2 * (e & 1) + 1], __uint_as_float(w[e] << 16),
+          __uint_as_float(w[e] & 0xffff0000u));
+  return (s[0] + s[1]) + (s[2] + s[3]);
 }
 
 struct RowState {
-  float m, la, lt;
+  float m;        // reference
+  float la, lt;   // sums over all keys, over the text keys
+  float dr;       // what rounding P to bf16 added to the row's large halves
 };
 
+// One half of the rows' key tile (the whole warp): exponentials, sums and P
+// against the rows' references.  When a row's sum passes kJump (its first
+// keys, a term far above the reference, NaN) that row takes the half's maximum
+// as its reference (at a row's first keys the whole key tile's: t_next is the
+// other half's S columns), and the warp's exponentials are taken once more; the
+// other rows' come out the same.
+// A term that dominates its row and is not a power of two is rounded in P and
+// would carry that error into O / la whole: where some row's sum passes kBig
+// (`big`, uniform), the caller adds to dr the difference between P's sum and the
+// exact one, and O is divided by la + dr, in which it cancels.
+// Returns the factor that the row's earlier sums (and O) were rescaled by;
+// `moved`, uniform: some row's is not 1.
+__device__ __forceinline__ float softmax_half(const uint32_t (&a)[32], const uint32_t (&b)[32],
+                                              uint32_t (&w)[32], int key0, int Nk, int L, float c,
+                                              RowState& st, float& sum, bool& moved, bool& big,
+                                              uint32_t t_next) {
+  // uniform: all 64 keys valid and on one side of the text's end
+  const bool plain = key0 + kHalf <= Nk && (key0 >= L || key0 + kHalf <= L);
+  float text, f = 1.f;
+  if (plain)
+    exp_half<false>(a, b, w, key0, Nk, L, c, st.m, sum, text);
+  else
+    exp_half<true>(a, b, w, key0, Nk, L, c, st.m, sum, text);
+  big = __any_sync(0xffffffffu, !(sum < kBig));
+  moved = false;
+  if (big) {
+    const bool over = !(sum < kJump);
+    moved = __any_sync(0xffffffffu, over);
+    if (moved) {
+      float next = -INFINITY;
+      if (t_next) {
+#pragma unroll 1
+        for (int k = 0; k < 2; ++k) {
+          uint32_t r[32];
+          tmem_ld32_wait(t_next + (uint32_t)(32 * k), r);
+#pragma unroll
+          for (int e = 0; e < 32; ++e)
+            if (key0 + kHalf + 32 * k + e < Nk) next = fmaxf(next, __uint_as_float(r[e]));
+        }
+      }
+      if (over) {
+        const float mx = plain ? half_max<false>(a, b, key0, Nk) : half_max<true>(a, b, key0, Nk);
+        const float m = fmaxf(st.m, fmaxf(mx, next) * c);
+        f = ex2(st.m - m);
+        st.la *= f;
+        st.lt *= f;
+        st.dr *= f;
+        st.m = m;
+      }
+      if (plain)
+        exp_half<false>(a, b, w, key0, Nk, L, c, st.m, sum, text);
+      else
+        exp_half<true>(a, b, w, key0, Nk, L, c, st.m, sum, text);
+    }
+  }
+  st.la += sum;
+  st.lt += text;
+  return f;
+}
+
 // Indices of a key tile's K and V loads in the ring: the load order is the
-// order the MMAs consume them, K_0, K_1, V_0, K_2, V_1, ... (S of the next
-// key tile is issued before P V of this one).  The K slot after the last
-// key tile is left unused.
-__device__ __forceinline__ int k_load(int g) { return g == 0 ? 0 : 2 * g - 1; }
-__device__ __forceinline__ int v_load(int g) { return 2 * g + 2; }
+// order the MMAs consume them.
+__device__ __forceinline__ int k_load(int g) { return 2 * g; }
+__device__ __forceinline__ int v_load(int g) { return 2 * g + 1; }
 
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -247,7 +309,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   uint8_t* sStage = sKV + C::kKVBytes;   // O staging, one 64-column block per tile
   Bars* bars = reinterpret_cast<Bars*>(sStage + kStageBytes);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int n_my = (p.n_units - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
   if (n_my <= 0) return;   // block-uniform
   const int G = n_my * p.n_kt;   // key tiles this CTA processes (all its units)
@@ -261,11 +323,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       mbar_init(&bars->q_full[t], 1);
       mbar_init(&bars->q_empty[t], 1);
       mbar_init(&bars->s_full[t], 1);
-      mbar_init(&bars->s_empty[t], 4);    // the tile's 4 softmax warps
-      mbar_init(&bars->p_full[t], 4);
-      mbar_init(&bars->pv_done[t], 1);
+      mbar_init(&bars->p_full[t][0], 4);   // the tile's 4 softmax warps
+      mbar_init(&bars->p_full[t][1], 4);
+      mbar_init(&bars->pv_half[t], 1);
       mbar_init(&bars->o_full[t], 1);
       mbar_init(&bars->o_empty[t], 4);
+      mbar_init(&bars->turn[t], 1);
       mbar_init(&bars->drain[t], 1);
     }
     for (int s = 0; s < C::kStages; ++s) {
@@ -293,134 +356,165 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     h = bh - b * p.H;
   };
 
-  if (warp == 0) {
+  if (warp < 4) {
+    // 128 x 88 + 256 x 208 = 384 x 168, what the block was launched with
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
     // ------------------------------------------------------ TMA producer --
-    if (lane == 0) {
+    if (warp == 0) {
       bool ok = true;
-      int last[C::kStages];   // the latest load armed on each stage, -1 = none
-      for (int s = 0; s < C::kStages; ++s) last[s] = -1;
+      int loads = 0;                 // K and V tiles armed so far, ring position
       int q_armed = 0, q_unit = 0;   // Q tiles armed for unit q_unit
+      int b, h, qp;
       auto load_q = [&](int ui, int t) {
-        int b, h, qp;
-        unit_coords((int)blockIdx.x + ui * (int)gridDim.x, b, h, qp);
         if (ui > 0)
           ok = mbar_wait_bounded(&bars->q_empty[t], (uint32_t)((ui - 1) & 1), abort_flag, p.status);
+        ok = __all_sync(0xffffffffu, ok);
         if (!ok) return;
-        if (q_unit != ui) { q_unit = ui; q_armed = 0; }
-        mbar_arrive_expect_tx(&bars->q_full[t], C::kTileBytes);
-        for (int cb = 0; cb < C::kCB; ++cb)
-          tma_load_4d(sQ + t * C::kTileBytes + cb * (kBM * 128), &tmQ, cb * 64,
-                      qp * kUnitRows + t * kBM, h, b, &bars->q_full[t]);
-        ++q_armed;
-      };
-      // load number idx of the ring: key tile g's K (is_k) or V
-      auto load_kv = [&](int idx, bool is_k, int g) {
-        int b, h, qp;
-        unit_coords((int)blockIdx.x + (g / p.n_kt) * (int)gridDim.x, b, h, qp);
-        const int kt = g - (g / p.n_kt) * p.n_kt;
-        const int stage = idx % C::kStages;
-        const uint32_t ph = (uint32_t)((idx / C::kStages) & 1);
-        ok = mbar_wait_bounded(&bars->kv_empty[stage], ph ^ 1u, abort_flag, p.status);
-        if (!ok) return;
-        mbar_arrive_expect_tx(&bars->kv_full[stage], C::kTileBytes);
-        for (int cb = 0; cb < C::kCB; ++cb)
-          tma_load_4d(sKV + stage * C::kTileBytes + cb * (kBM * 128), is_k ? &tmK : &tmV, cb * 64,
-                      kt * kBN, h, b, &bars->kv_full[stage]);
-        last[stage] = idx;
-      };
-      load_q(0, 0);
-      if (ok) load_kv(k_load(0), true, 0);
-      if (ok) load_q(0, 1);
-      for (int g = 0; g < G && ok; ++g) {
-        const int gn = g + 1;
-        if (gn < G) {
-          if (gn % p.n_kt == 0) {   // the next unit's Q tiles before its first K tile
-            load_q(gn / p.n_kt, 0);
-            if (ok) load_q(gn / p.n_kt, 1);
-          }
-          if (ok) load_kv(k_load(gn), true, gn);
+        q_armed = t + 1;
+        q_unit = ui;
+        if (elect_one()) {
+          mbar_arrive_expect_tx(&bars->q_full[t], C::kTileBytes);
+          for (int cb = 0; cb < C::kCB; ++cb)
+            tma_load_4d(sQ + t * C::kTileBytes + cb * (kBM * 128), &tmQ, cb * 64,
+                        qp * kUnitRows + t * kBM, h, b, &bars->q_full[t]);
         }
-        if (ok) load_kv(v_load(g), false, g);
+        __syncwarp();
+      };
+      // the ring's next load: key tile kt of the unit
+      auto load_kv = [&](const CUtensorMap* map, int kt) {
+        const int stage = loads % C::kStages;
+        const uint32_t ph = (uint32_t)((loads / C::kStages) & 1);
+        ok = mbar_wait_bounded(&bars->kv_empty[stage], ph ^ 1u, abort_flag, p.status);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) return;
+        ++loads;
+        if (elect_one()) {
+          mbar_arrive_expect_tx(&bars->kv_full[stage], C::kTileBytes);
+          for (int cb = 0; cb < C::kCB; ++cb)
+            tma_load_4d(sKV + stage * C::kTileBytes + cb * (kBM * 128), map, cb * 64, kt * kBN, h, b,
+                        &bars->kv_full[stage]);
+        }
+        __syncwarp();
+      };
+      for (int ui = 0; ui < n_my && ok; ++ui) {
+        unit_coords((int)blockIdx.x + ui * (int)gridDim.x, b, h, qp);
+        load_q(ui, 0);
+        if (ok && ui > 0) load_q(ui, 1);
+        if (ok) load_kv(&tmK, 0);
+        if (ok && ui == 0) load_q(ui, 1);   // the first K tile ahead of it at the start
+        if (ok) load_kv(&tmV, 0);
+        for (int kt = 1; kt < p.n_kt && ok; ++kt) {
+          load_kv(&tmK, kt);
+          if (ok) load_kv(&tmV, kt);
+        }
       }
       if (!ok) {
         // drain the copies still in flight before the CTA exits
         for (int t = 0; t < q_armed; ++t)
           mbar_wait_bounded(&bars->q_full[t], (uint32_t)(q_unit & 1), nullptr, p.status);
-        for (int s = 0; s < C::kStages; ++s)
-          if (last[s] >= 0)
-            mbar_wait_bounded(&bars->kv_full[s], (uint32_t)((last[s] / C::kStages) & 1), nullptr,
-                              p.status);
+        for (int i = loads > C::kStages ? loads - C::kStages : 0; i < loads; ++i)
+          mbar_wait_bounded(&bars->kv_full[i % C::kStages], (uint32_t)((i / C::kStages) & 1),
+                            nullptr, p.status);
       }
     }
-  } else if (warp == 1 || warp == 2) {
     // -------------------------------------------------------- MMA issuers --
-    // Key tile g: S_t(g) = Q_t K_g^T into the S buffer both tiles share, as
-    // soon as the other tile's softmax has loaded the S before it (S_0(g)
-    // after S_1(g-1), S_1(g) after S_0(g)); then O_t += P_t(g-1) V_(g-1) with
-    // P_t from tensor memory once the softmax has written it.  The next S so
-    // runs on the tensor pipe while the softmax works on this one.
-    const int t = warp - 1;
-    if (lane == 0) {
-      bool ok = true;
+    // S_t(0); then per key tile g a turn: the two halves of O_t += P_t(g) V_g
+    // and S_t(g+1) behind them.  The tensor pipe runs one thread's products in
+    // the order they were issued, so S_t(g+1) may overwrite P_t(g).
+    if (warp == 1 || warp == 2) {
+      const int t = warp - 1;
       const uint32_t q_lo = sw128_desc_lo(sQ + t * C::kTileBytes);
       const uint32_t kv_lo0 = sw128_desc_lo(sKV);
       const uint32_t v_lo0 = sw128_mn_desc_lo(sKV, kBM * 128);
       const uint32_t d_hi = sw128_desc_hi();
-      const uint32_t tS = tmem + (uint32_t)kColS;
-      const uint32_t tP = tmem + (uint32_t)(kColP + t * (kBN / 2));
+      const uint32_t tS = tmem + (uint32_t)(kColS + t * kBN);
       const uint32_t tO = tmem + (uint32_t)(kColO + t * D);
-      for (int gi = 0; gi <= G && ok; ++gi) {
-        if (gi < G) {
-          const int ui = gi / p.n_kt, j = gi - ui * p.n_kt;
-          const int lk = k_load(gi), sk = lk % C::kStages;
-          ok = mbar_wait_bounded(&bars->kv_full[sk], (uint32_t)((lk / C::kStages) & 1), abort_flag, p.status);
-          if (ok && j == 0)
-            ok = mbar_wait_bounded(&bars->q_full[t], (uint32_t)(ui & 1), abort_flag, p.status);
-          // the shared S buffer: the previous S in the order S_0(0), S_1(0),
-          // S_0(1), ... has been loaded by its softmax
-          if (ok && t == 0 && gi > 0)
-            ok = mbar_wait_bounded(&bars->s_empty[1], (uint32_t)((gi - 1) & 1), abort_flag, p.status);
-          if (ok && t == 1)
-            ok = mbar_wait_bounded(&bars->s_empty[0], (uint32_t)(gi & 1), abort_flag, p.status);
-          if (!ok) break;
-          fence_after();
-          const uint32_t k_lo = kv_lo0 + (uint32_t)((sk * C::kTileBytes) >> 4);
+      bool ok = true;
+      auto wait = [&](uint64_t* bar, int phase) {
+        if (ok) ok = mbar_wait_bounded(bar, (uint32_t)(phase & 1), abort_flag, p.status);
+      };
+      int s_u = 0;   // unit of the next S
+      auto issue_s = [&](int lk, bool last) {   // lk: the K tile's number in the ring
+        const uint32_t k_lo = kv_lo0 + (uint32_t)(((lk % C::kStages) * C::kTileBytes) >> 4);
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk) {
             const uint32_t off = (uint32_t)(((kk >> 2) * (kBM * 128) + (kk & 3) * 32) >> 4);
             mma_ss(tS, q_lo + off, k_lo + off, d_hi, kIdescS, kk > 0 ? 1u : 0u);
           }
           mma_commit(&bars->s_full[t]);
-          mma_commit(&bars->kv_empty[sk]);
-          if (j == p.n_kt - 1) mma_commit(&bars->q_empty[t]);
+          mma_commit(&bars->kv_empty[lk % C::kStages]);
+          if (last) mma_commit(&bars->q_empty[t]);
         }
-        if (gi > 0) {
-          const int g = gi - 1;
-          const int ug = g / p.n_kt, jg = g - ug * p.n_kt;
-          const int lv = v_load(g), sv = lv % C::kStages;
-          ok = mbar_wait_bounded(&bars->p_full[t], (uint32_t)(g & 1), abort_flag, p.status);
-          if (ok)
-            ok = mbar_wait_bounded(&bars->kv_full[sv], (uint32_t)((lv / C::kStages) & 1), abort_flag, p.status);
-          if (ok && jg == 0 && ug > 0)   // the epilogue has read the previous unit's O_t
-            ok = mbar_wait_bounded(&bars->o_empty[t], (uint32_t)((ug - 1) & 1), abort_flag, p.status);
+        __syncwarp();
+      };
+      auto pass_turn = [&]() {
+        if (lane == 0) mbar_arrive(&bars->turn[t ^ 1]);
+      };
+      wait(&bars->kv_full[0], 0);
+      wait(&bars->q_full[t], 0);
+      if (t == 1) wait(&bars->turn[1], 0);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) {
+        issue_s(k_load(0), p.n_kt == 1);
+        pass_turn();
+      }
+      int v_j = 0, v_u = 0;   // key tile within the unit, and unit, of P V
+      for (int g = 0; g < G && ok; ++g) {
+        const int lv = v_load(g), lk = k_load(g + 1);
+        const bool more = g + 1 < G, next_unit = v_j == p.n_kt - 1;
+        // waited for while the other tile has its turn
+        if (v_j == 0 && v_u > 0) wait(&bars->o_empty[t], v_u - 1);   // O_t of the previous unit is read
+        wait(&bars->kv_full[lv % C::kStages], lv / C::kStages);
+        if (more && !next_unit) wait(&bars->kv_full[lk % C::kStages], lk / C::kStages);
+        wait(&bars->p_full[t][0], g);
+        wait(&bars->turn[t], t == 0 ? g : g + 1);
+        const uint32_t v_lo = v_lo0 + (uint32_t)(((lv % C::kStages) * C::kTileBytes) >> 4);
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          if (hf == 1) wait(&bars->p_full[t][1], g);
+          ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           fence_after();
-          const uint32_t v_lo = v_lo0 + (uint32_t)((sv * C::kTileBytes) >> 4);
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < kBN / 16; ++kk)   // 16 keys: 8 P columns, 16 V rows
-            mma_ts(tO, tP + (uint32_t)(kk * 8), v_lo + (uint32_t)((kk * 16 * 128) >> 4), d_hi,
-                   C::kIdescPV, (jg > 0 || kk > 0) ? 1u : 0u);
-          mma_commit(&bars->pv_done[t]);
-          mma_commit(&bars->kv_empty[sv]);
-          if (jg == p.n_kt - 1) mma_commit(&bars->o_full[t]);
+            for (int k4 = 0; k4 < kHalf / 16; ++k4) {   // 16 keys: 8 P columns, 16 V rows
+              const int kk = hf * (kHalf / 16) + k4;
+              mma_ts(tO, tS + (uint32_t)(kk * 8), v_lo + (uint32_t)((kk * 16 * 128) >> 4), d_hi,
+                     C::kIdescPV, (v_j > 0 || kk > 0) ? 1u : 0u);
+            }
+            if (hf == 0) {
+              mma_commit(&bars->pv_half[t]);
+            } else {
+              mma_commit(&bars->kv_empty[lv % C::kStages]);
+              if (next_unit) mma_commit(&bars->o_full[t]);
+            }
+          }
+          __syncwarp();
         }
+        if (!ok) break;
+        if (more) {
+          if (next_unit) {
+            ++s_u;
+            wait(&bars->q_full[t], s_u);
+            wait(&bars->kv_full[lk % C::kStages], lk / C::kStages);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+          }
+          const int s_j = next_unit ? 0 : v_j + 1;
+          issue_s(lk, s_j == p.n_kt - 1);
+        }
+        pass_turn();
+        if (next_unit) { v_j = 0; ++v_u; } else { ++v_j; }
       }
       // all issued MMAs complete before tensor memory is released
-      mma_commit(&bars->drain[t]);
+      if (elect_one()) mma_commit(&bars->drain[t]);
+      __syncwarp();
       mbar_wait_bounded(&bars->drain[t], 0, nullptr, p.status);
     }
-  } else if (warp >= 4) {
+  } else {
     // --------------------------------------------- softmax and epilogue --
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
     const int t = (warp - 4) >> 2;
     const int quad = warp & 3;             // TMEM lane quadrant this warp may access
     const int rowt = quad * 32 + lane;     // row within the tile = TMEM lane
@@ -430,8 +524,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     auto tile_sync = [&]() { if (t == 0) bar_sync(1, 128); else bar_sync(2, 128); };
     auto tile_and = [&](bool v) { return t == 0 ? bar_and(1, 128, v) : bar_and(2, 128, v); };
     const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
-    const uint32_t tS = tmem + lane_off + (uint32_t)kColS;
-    const uint32_t tP = tmem + lane_off + (uint32_t)(kColP + t * (kBN / 2));
+    const uint32_t tS = tmem + lane_off + (uint32_t)(kColS + t * kBN);
     const uint32_t tO = tmem + lane_off + (uint32_t)(kColO + t * D);
     uint8_t* sSt = sStage + t * kStageTileBytes;
     const float c = p.c_log2;
@@ -440,80 +533,50 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     for (int ui = 0; ui < n_my; ++ui) {
       int b, h, qp;
       unit_coords((int)blockIdx.x + ui * (int)gridDim.x, b, h, qp);
-      RowState st{-INFINITY, 0.f, 0.f};
+      RowState st{-INFINITY, 0.f, 0.f, 0.f};
       for (int j = 0; j < p.n_kt; ++j, ++gi) {
         ok = ok && (*abort_flag == 0) &&
              mbar_wait_bounded(&bars->s_full[t], (uint32_t)(gi & 1), abort_flag, p.status);
         ok = __all_sync(0xffffffffu, ok);   // tcgen05.ld / st are warp-collective
-        if (ok) {
-          fence_after();
-          // the row's 128 S columns into registers; the S buffer is then free
-          // for the other tile's S
-          uint32_t r0[32], r1[32], r2[32], r3[32];
-          tmem_ld32(tS, r0);
-          tmem_ld32(tS + 32, r1);
-          tmem_ld32(tS + 64, r2);
-          tmem_ld32(tS + 96, r3);
-          tmem_wait32(r0);
-          tmem_wait32(r1);
-          tmem_wait32(r2);
-          tmem_wait32(r3);
+        if (!ok) continue;
+        fence_after();
+        // one body for both halves: 5 KB of straight-line code that stays in
+        // the instruction cache
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          uint32_t r0[32], r1[32], w[32];
+          tmem_ld64_wait(tS + (uint32_t)(h * kHalf), r0, r1);
+          bool moved, big;
+          float sum;
+          const float f = softmax_half(r0, r1, w, j * kBN + h * kHalf, p.Nk, p.L, c, st, sum, moved,
+                                       big, j + h == 0 ? tS + (uint32_t)kHalf : 0u);
+          if (moved && j + h > 0) {
+            // O_t holds the products before this half (S_t complete: all of the
+            // earlier tiles'; the first half's is waited for)
+            if (h == 1) {
+              ok = mbar_wait_bounded(&bars->pv_half[t], (uint32_t)(gi & 1), abort_flag, p.status);
+              ok = __all_sync(0xffffffffu, ok);
+              if (!ok) break;
+              fence_after();
+            }
+            rescale_o<D>(tO, f);
+          }
+          // P over S columns that are in registers
+          tmem_st32(tS + (uint32_t)(h * (kHalf / 2)), w);
+          tmem_wait_st();
           fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&bars->s_empty[t]);
-          const int key0 = j * kBN;
-          float mx;
-          if (key0 + kBN <= p.Nk)
-            mx = fmaxf(fmaxf(chunk_max<true>(r0, 0, 0), chunk_max<true>(r1, 0, 0)),
-                       fmaxf(chunk_max<true>(r2, 0, 0), chunk_max<true>(r3, 0, 0)));
-          else
-            mx = fmaxf(fmaxf(chunk_max<false>(r0, key0, p.Nk), chunk_max<false>(r1, key0 + 32, p.Nk)),
-                       fmaxf(chunk_max<false>(r2, key0 + 64, p.Nk),
-                             chunk_max<false>(r3, key0 + 96, p.Nk)));
-          const float mt = mx * c;
-          const bool up = mt > st.m + kTau;   // the row's first tile, or 2^8 above its maximum
-          float f = 1.f;
-          if (up) {
-            f = ex2(st.m - mt);
-            st.la *= f;
-            st.lt *= f;
-            st.m = mt;
-          }
-          // the numerators (bf16 pairs) while the previous PV product may
-          // still be reading P_t; the kind is uniform over the warp
-          if (key0 + kBN <= p.Nk && key0 >= p.L)
-            exp_tile<0>(r0, r1, r2, r3, key0, p.Nk, p.L, c, st.m, st.la, st.lt);
-          else if (key0 + kBN <= p.Nk && key0 + kBN <= p.L)
-            exp_tile<1>(r0, r1, r2, r3, key0, p.Nk, p.L, c, st.m, st.la, st.lt);
-          else
-            exp_tile<2>(r0, r1, r2, r3, key0, p.Nk, p.L, c, st.m, st.la, st.lt);
-          // P_t(gi - 1) has been read by its PV product and O_t holds it
-          if (gi > 0) {
-            bool w = mbar_wait_bounded(&bars->pv_done[t], (uint32_t)((gi - 1) & 1), abort_flag, p.status);
-            ok = __all_sync(0xffffffffu, w);
-          }
-          if (ok) {
-            // P_t into tensor memory: column c of the row holds keys 2c, 2c + 1
-            tmem_st_p(tP, r0);
-            tmem_st_p(tP + 16, r1);
-            tmem_st_p(tP + 32, r2);
-            tmem_st_p(tP + 48, r3);
-            // the warp rescales its O rows together when any of them moved
-            // (f = 1 leaves a row unchanged)
-            if (j > 0 && __any_sync(0xffffffffu, up)) rescale_o<D>(tO, f);
-            tmem_wait_st();
-            fence_before();
-          }
+          if (lane == 0) mbar_arrive(&bars->p_full[t][h]);
+          // behind the hand-over: nothing waits for it
+          if (big) st.dr += rounded_sum(w) - sum;
         }
-        __syncwarp();
-        if (ok && lane == 0) mbar_arrive(&bars->p_full[t]);
       }
       // ---- epilogue: O / l -> bf16 -> swizzled staging, 64 columns at a
       // time -> TMA store
       ok = ok && (*abort_flag == 0) &&
            mbar_wait_bounded(&bars->o_full[t], (uint32_t)(ui & 1), abort_flag, p.status);
       ok = __all_sync(0xffffffffu, ok);
-      const float inv = 1.f / st.la;
+      const float inv = 1.f / (st.la + st.dr);
       const int row0 = qp * kUnitRows + t * kBM;
 #pragma unroll 1
       for (int cb = 0; cb < C::kCB; ++cb) {
@@ -522,8 +585,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll 1
           for (int k = 0; k < 2; ++k) {
             uint32_t r[32];
-            tmem_ld32(tO + 64 * cb + 32 * k, r);
-            tmem_wait32(r);
+            tmem_ld32_wait(tO + (uint32_t)(64 * cb + 32 * k), r);
             uint32_t w[16];
 #pragma unroll
             for (int e = 0; e < 16; ++e)

@@ -147,37 +147,18 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t base, uint32_t cols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols));
 }
 
-#define AVITS_R8(b) "=r"(r[b]), "=r"(r[b + 1]), "=r"(r[b + 2]), "=r"(r[b + 3]), \
-                    "=r"(r[b + 4]), "=r"(r[b + 5]), "=r"(r[b + 6]), "=r"(r[b + 7])
-#define AVITS_W8(b) "+r"(r[b]), "+r"(r[b + 1]), "+r"(r[b + 2]), "+r"(r[b + 3]), \
-                    "+r"(r[b + 4]), "+r"(r[b + 5]), "+r"(r[b + 6]), "+r"(r[b + 7])
 #define AVITS_I8(b) "r"(r[b]), "r"(r[b + 1]), "r"(r[b + 2]), "r"(r[b + 3]), \
                     "r"(r[b + 4]), "r"(r[b + 5]), "r"(r[b + 6]), "r"(r[b + 7])
-
-// 16 / 32 consecutive 32-bit columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-      "%11, %12, %13, %14, %15}, [%16];"
-      : AVITS_R8(0), AVITS_R8(8)
-      : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-      "%11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
-      "%28, %29, %30, %31}, [%32];"
-      : AVITS_R8(0), AVITS_R8(8), AVITS_R8(16), AVITS_R8(24)
-      : "r"(taddr));
-}
 
 #define AVITS_O8(r, b) "=r"(r[b]), "=r"(r[b + 1]), "=r"(r[b + 2]), "=r"(r[b + 3]), \
                        "=r"(r[b + 4]), "=r"(r[b + 5]), "=r"(r[b + 6]), "=r"(r[b + 7])
 
-// Loads with the wait in the same statement, for the softmax loops: a separate
-// wait has to name the registers as in-out operands to keep their uses behind
-// it, and the compiler then copied them (4 % of the spatial kernel's time).
-// 32 consecutive columns, complete on return.
+// Columns of this thread's TMEM lane into registers, complete on return.  The
+// wait is in the same statement: a separate one has to name the registers as
+// in-out operands to keep their uses behind it, and the compiler then copied
+// them (7 % more instructions in the attention kernel, 178 -> 165 us; 4 % of
+// the spatial kernel's time).
+// 32 consecutive columns.
 __device__ __forceinline__ void tmem_ld32_wait(uint32_t taddr, uint32_t (&a)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
@@ -188,26 +169,22 @@ __device__ __forceinline__ void tmem_ld32_wait(uint32_t taddr, uint32_t (&a)[32]
       : "r"(taddr)
       : "memory");
 }
-
-// Completes the thread's outstanding tcgen05.ld; the registers are tied to
-// the wait so that no use can be scheduled before it.
-__device__ __forceinline__ void tmem_wait(uint32_t (&r)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" : AVITS_W8(0), AVITS_W8(8) : : "memory");
-}
-__device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : AVITS_W8(0), AVITS_W8(8), AVITS_W8(16), AVITS_W8(24)
-               :
-               : "memory");
-}
-
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+// 64 consecutive columns (a: the first 32).
+__device__ __forceinline__ void tmem_ld64_wait(uint32_t taddr, uint32_t (&a)[32], uint32_t (&b)[32]) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-      "%11, %12, %13, %14, %15, %16};" ::"r"(taddr),
-      AVITS_I8(0), AVITS_I8(8)
+      "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+      "%11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
+      "%28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, "
+      "%45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, "
+      "%62, %63}, [%64];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : AVITS_O8(a, 0), AVITS_O8(a, 8), AVITS_O8(a, 16), AVITS_O8(a, 24), AVITS_O8(b, 0),
+        AVITS_O8(b, 8), AVITS_O8(b, 16), AVITS_O8(b, 24)
+      : "r"(taddr)
       : "memory");
 }
+
+// 32 registers to consecutive columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
@@ -250,15 +227,6 @@ __device__ __forceinline__ void fadd2(float& s0, float& s1, float e0, float e1) 
       "add.rn.f32x2 ra, ra, rb;\n\tmov.b64 {%0, %1}, ra;\n\t}"
       : "+f"(s0), "+f"(s1)
       : "f"(e0), "f"(e1));
-}
-
-// (a0, a1) *= b on a packed pair.
-__device__ __forceinline__ void fmul2(float& a0, float& a1, float b) {
-  asm("{\n\t.reg .b64 ra, rb;\n\t"
-      "mov.b64 ra, {%0, %1};\n\tmov.b64 rb, {%2, %2};\n\t"
-      "mul.rn.f32x2 ra, ra, rb;\n\tmov.b64 {%0, %1}, ra;\n\t}"
-      : "+f"(a0), "+f"(a1)
-      : "f"(b));
 }
 
 // Two fp32 -> one bf16x2 word (round to nearest even), lo in the low half.
