@@ -537,6 +537,8 @@ fuse_select_kernel(const SelArgs g) {
 // SMs) while the copy lands; part 0 writes the selection outputs; finally
 // each warp upsamples its tokens from shared memory.  No CTA waits for
 // another.
+// One CTA per SM is all the grid asks for; told so, the compiler gives the
+// bilinear instances the registers they use (batch 16 13.2 -> 11.5 us).
 template <int kThreads, int kRegKeys, typename T, bool kBilinear>
 __global__ void __launch_bounds__(kThreads, 1)
 select_upsample_kernel(const SelArgs g, const UpsampleArgs<T> u, int parts, int stage_rows) {

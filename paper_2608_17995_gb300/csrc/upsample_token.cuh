@@ -64,6 +64,10 @@ struct SharedRows {
 // are taken from the child's side: index 0 = towards the neighbour, 1 = the
 // parent's pixel, 2 = inside the own token; the weights are symmetric, so the
 // sums are those of the general path, term for term.
+// Bound by instructions and the latency of a token's chain (a warp per token),
+// not by bytes; a lane per (child, channel) read nine scalars for each.  One
+// launch with the selection, 32 x 32 grids of 16 bf16 channels, us: batch 1 5.6 ->
+// 5.2, 16 13.5 -> 11.5, 64 34.4 -> 29.5.
 template <typename T, typename Src>
 __device__ __forceinline__ uint4 bilinear_child(const Src& rows, int b_elem, int gh, int gw, int y,
                                                 int x, int a, int b, int j) {
