@@ -427,7 +427,8 @@ merge_bilinear_kernel(const T* __restrict__ mixed, int B, int N, const int32_t* 
 
 // Bilinear merge, pass 2, for tokens of whole 16-byte pieces: a CTA takes a tile
 // of 16 x 16 cells and two pieces (32 bytes) of the channels.  It loads the
-// cell map of the tile and four cells around it, turns every cell of the tile
+// cell map of the tile and four cells around it (an entry of the tile that no
+// token of this call covers is a hole: reported, zeros), turns every cell of the tile
 // and the ring next to it into its level-1 pixel (one 16-byte load: a span-2
 // token's pixel, or the average of a span-1 token's four) in shared memory,
 // and writes the cells from the 3 x 3 level-1 pixels around them; span-1 cells
@@ -437,11 +438,13 @@ merge_bilinear_kernel(const T* __restrict__ mixed, int B, int N, const int32_t* 
 // order of operations.  What bounds it: the chain map - token - shared memory -
 // cell at a few CTAs per SM, then the copies.  us of the two kernels, against a
 // thread per (cell, channel) behind a fill and an atomic scatter, bf16, 64 x 64
-// cells of 16 channels: batch 1 8.4 -> 6.5, 16 31.3 -> 12.8, 64 102 -> 33.7;
-// batch 32 with spans 1, 2 and 4 2606 -> 29.8 (a value of level 2 was pooled
-// anew by every thread that drew on it).  Left out: a thread per 2 x 2 cells
-// with the neighbourhood in registers, 10.5 at batch 16 but 5580 with span 4;
-// three pieces of a thread in flight 13.2.
+// cells of 16 channels: batch 1 8.4 -> 6.3, 16 31.3 -> 11.5, 64 102 -> 31.4; batch
+// 32 with spans 1, 2 and 4 2606 -> 28.4 (a value of level 2 was pooled anew by
+// every thread that drew on it).  A cell's token is checked once, where the map
+// is loaded (by each piece's thread: 12.8 at batch 16).  Left out: a thread per
+// 2 x 2 cells with the neighbourhood in registers, 10.5 at batch 16 but 5580 with
+// span 4; three pieces of a thread in flight (13.2 against 12.8); four pieces per
+// CTA (12.9); the pieces' planes 16 banks apart (12.4).
 constexpr int kTile = 16;
 constexpr int kHalo = 4;                        // cells around the tile that level 2 can draw on
 constexpr int kReg = kTile + 2 * kHalo;
@@ -481,6 +484,10 @@ merge_bilinear_tile_kernel(const T* __restrict__ mixed, int N, const int32_t* __
     if (Y >= 0 && Y < fh && X >= 0 && X < fw) {
       e = mapb[(int64_t)Y * fw + X];
       if (e >= 0 && map_tok(e) >= N) e = -1;
+      if (r >= kHalo && r < kHalo + kTile && c >= kHalo && c < kHalo + kTile) {
+        e = live_entry(e, N, posb, spanb, Y, X);
+        if (e < 0) raise_status(status, AVITS_ERR_COVERAGE);
+      }
     }
     smap[r][c] = e;
     wide = wide || (e >= 0 && map_lvl(e) >= 2 && r >= kHalo - 1 && r <= kHalo + kTile &&
@@ -500,19 +507,13 @@ merge_bilinear_tile_kernel(const T* __restrict__ mixed, int N, const int32_t* __
     const int pc = i % kTilePieces, q = i / kTilePieces;
     const int r = first + q / side, c = first + q % side;
     if (pc >= npc) continue;
-    int32_t e = smap[r][c];
+    const int32_t e = smap[r][c];
     const int Y = Y0 - kHalo + r, X = X0 - kHalo + c;
     const bool mine = r >= kHalo && r < kHalo + kTile && c >= kHalo && c < kHalo + kTile &&
                       Y < fh && X < fw;
     const uint4 w = e >= 0 ? piece(e, pc) : make_uint4(0u, 0u, 0u, 0u);
-    if (mine && live_entry(e, N, posb, spanb, Y, X) < 0) {
-      raise_status(status, AVITS_ERR_COVERAGE);
-      write(Y, X, pc, make_uint4(0u, 0u, 0u, 0u));
-      smap[r][c] = -1;   // this cell's other piece reads no token, or found so as well
-      e = -1;
-    }
     const int lvl = e >= 0 ? map_lvl(e) : -1;
-    if (mine && lvl == 0) write(Y, X, pc, w);
+    if (mine && lvl <= 0) write(Y, X, pc, w);   // a span-1 cell, or zeros in a hole
     float p[kCh][4];
     Chunk<T>::unpack(w, p);
 #pragma unroll
