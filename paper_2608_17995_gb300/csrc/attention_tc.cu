@@ -58,12 +58,13 @@
 // a clock), two halves of load, exponentials and store (~1600), waits (~200),
 // the second half's PV product; the pipe itself needs ~2290 clocks per key tile
 // for both tiles.  24 heads of 128, one image at 1024^2 (1536 x 1536): 27.2 ->
-// 25.9 us; at 2048^2 (4608 x 4608): 197 -> 177 us (1478 TFLOP/s, 0.78 of the
-// measured bf16 peak); batch 2: 395 -> 348 us, 413 -> 373 where logits rise along
+// 26.2 us; at 2048^2 (4608 x 4608): 197 -> 178 us (1462 TFLOP/s, 0.76 of the
+// measured bf16 peak); batch 2: 395 -> 354 us, 413 -> 375 where logits rise along
 // the keys.  Without the care for P's rounding (kBig) 23.8 / 164 / 327 us, but the
 // error of O against 64 bits was then 3 to 6 % above the earlier kernel's; with
-// it 1 to 2 % below (kBig 2^8: equal, 2^6: 5 % below, 355 us).  References moved
-// from 2^9 on instead: equal, 370 us.
+// it 1 to 4 % below (from 2^7 on: 0.5 to 2 % below, 25.7 / 175 / 349 us; 2^5: 1 to
+// 6 %, 362 us; always: 7 to 11 %, 385 us).  References moved from 2^9 on instead:
+// equal, 370 us.
 // Measured and left out at 2048^2 (against 164): 16 softmax warps, two threads
 // per row (186 us); S in 64-key products with the next step's S behind this
 // step's PV (186: half-width products read Q twice); the turn passed before the
@@ -90,7 +91,7 @@ constexpr int kThreads = 12 * 32;
 constexpr int kTmemCols = 512;
 constexpr int kHalf = kBN / 2;      // keys the softmax handles at a time
 constexpr float kJump = 0x1p16f;    // a half's sum from which the reference moves
-constexpr float kBig = 0x1p7f;      // and from which P's rounding is made up for
+constexpr float kBig = 0x1p6f;      // and from which P's rounding is made up for
 constexpr uint32_t kIdescS = idesc_bf16(kBM, kBN, false);
 
 template <int D>
@@ -237,9 +238,10 @@ struct RowState {
 // other half's S columns), and the warp's exponentials are taken once more; the
 // other rows' come out the same.
 // A term that dominates its row and is not a power of two is rounded in P and
-// would carry that error into O / la whole: where some row's sum passes kBig
-// (`big`, uniform), the caller adds to dr the difference between P's sum and the
-// exact one, and O is divided by la + dr, in which it cancels.
+// would carry that error into O / la whole: where the row's own sum, before any
+// such move, passed kBig (`big`), the caller adds to dr the difference between
+// P's sum and the exact one, and O is divided by la + dr, in which it cancels.  No
+// row's result depends on another row of its warp.
 // Returns the factor that the row's earlier sums (and O) were rescaled by;
 // `moved`, uniform: some row's is not 1.
 __device__ __forceinline__ float softmax_half(const uint32_t (&a)[32], const uint32_t (&b)[32],
@@ -253,9 +255,9 @@ __device__ __forceinline__ float softmax_half(const uint32_t (&a)[32], const uin
     exp_half<false>(a, b, w, key0, Nk, L, c, st.m, sum, text);
   else
     exp_half<true>(a, b, w, key0, Nk, L, c, st.m, sum, text);
-  big = __any_sync(0xffffffffu, !(sum < kBig));
+  big = !(sum < kBig);
   moved = false;
-  if (big) {
+  if (__any_sync(0xffffffffu, big)) {
     const bool over = !(sum < kJump);
     moved = __any_sync(0xffffffffu, over);
     if (moved) {
@@ -568,7 +570,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           __syncwarp();
           if (lane == 0) mbar_arrive(&bars->p_full[t][h]);
           // behind the hand-over: nothing waits for it
-          if (big) st.dr += rounded_sum(w) - sum;
+          if (__any_sync(0xffffffffu, big)) {
+            const float d = rounded_sum(w) - sum;
+            if (big) st.dr += d;
+          }
         }
       }
       // ---- epilogue: O / l -> bf16 -> swizzled staging, 64 columns at a
