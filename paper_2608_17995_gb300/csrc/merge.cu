@@ -17,7 +17,8 @@
 // leaves a hole that pass 2 finds), then clears the word.  The map needs no
 // clearing between calls.
 // Bilinear (spans 1, 2 and 4): pass 1 as above with each entry carrying the
-// token's level; in pass 2 span-1 cells are copied, coarser cells take the
+// token's level; in pass 2, where an entry that is no cover counts as a hole for
+// the cells around it as well, span-1 cells are copied, coarser cells take the
 // half-pixel-centred 2x bilinear resize of level 1 of the frame's pixel
 // pyramid (frame_map.cuh), refined first from level 2 inside span-4 tokens.
 // Algorithmic bytes: B*N*(T*elt + 12) read + B*fh*fw*T*elt written.
@@ -303,19 +304,16 @@ __global__ void merge_map_kernel(int B, int N, const int32_t* __restrict__ pos,
     }
 }
 
-// The four pixels of a cell from level-1 pixels around it: output pixel row
-// 2Y + a draws on level-1 rows (Y - 1, Y) for a = 0 and (Y, Y + 1) for a = 1
-// with weights (1/4, 3/4) / (3/4, 1/4), clamped at the frame edge by the
-// neighbourhood; columns likewise.  lv[u][v] is the cell's upper left
-// neighbour.
-template <int K>
-__device__ __forceinline__ void resize_cell(const float (&lv)[K][K], int u, int v, float (&r)[4]) {
+// The four pixels of a cell from the 3 x 3 level-1 pixels around it: output
+// pixel row 2Y + a draws on level-1 rows (Y - 1, Y) for a = 0 and (Y, Y + 1) for
+// a = 1 with weights (1/4, 3/4) / (3/4, 1/4), clamped at the frame edge by the
+// neighbourhood; columns likewise.
+__device__ __forceinline__ void resize_cell(const float (&lv)[3][3], float (&r)[4]) {
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int a = q >> 1, b = q & 1;
-    r[q] = bil_combine(lv[u + a][v + b], lv[u + a][v + b + 1], lv[u + a + 1][v + b],
-                       lv[u + a + 1][v + b + 1], a ? 0.75f : 0.25f, a ? 0.25f : 0.75f,
-                       b ? 0.75f : 0.25f, b ? 0.25f : 0.75f);
+    r[q] = bil_combine(lv[a][b], lv[a][b + 1], lv[a + 1][b], lv[a + 1][b + 1], a ? 0.75f : 0.25f,
+                       a ? 0.25f : 0.75f, b ? 0.75f : 0.25f, b ? 0.25f : 0.75f);
   }
 }
 
@@ -356,57 +354,54 @@ merge_scatter_kernel(int B, int N, const int32_t* __restrict__ pos,
   if (threadIdx.x == 0) count_cells(hdr, cta_cells, (unsigned long long)B * fh * fw, status);
 }
 
-// The entry of a cell if its token covers the cell in this call, else -1 (a
-// hole: the entry of an earlier call).
-__device__ __forceinline__ int32_t live_entry(int32_t e, int N, const int32_t* __restrict__ posb,
-                                              const int32_t* __restrict__ spanb, int Y, int X) {
-  if (e < 0) return -1;
-  const int t = map_tok(e), s = 1 << map_lvl(e);
-  if (t >= N || spanb[t] != s) return -1;
-  const int y = posb[t * 2], x = posb[t * 2 + 1];
-  return (Y & ~(s - 1)) == y && (X & ~(s - 1)) == x ? e : -1;
-}
+// What pass 1 left for a cell: its word and the place of the token that the
+// word names (token 0 where it names none of this call's; loaded at once, so that
+// a caller can have several in flight).
+struct CellWord {
+  int32_t e;
+  int s, y, x;
+  __device__ void place(int N, const int32_t* __restrict__ posb, const int32_t* __restrict__ spanb) {
+    const int t = e >= 0 && map_tok(e) < N ? map_tok(e) : 0;
+    s = spanb[t];
+    y = posb[t * 2];
+    x = posb[t * 2 + 1];
+  }
+  // The word if its token covers the cell in this call, else -1 (a hole: the
+  // word is what an earlier call, of either mode and of any token count, left
+  // there).  Only a word that passed here may be followed to a token.
+  __device__ int32_t live(int N, int fh, int fw, int Y, int X) const {
+    const bool ok = e >= 0 && map_lvl(e) <= kMaxMapLevel && map_tok(e) < N && s == 1 << map_lvl(e) &&
+                    (Y & ~(s - 1)) == y && (X & ~(s - 1)) == x && y + s <= fh && x + s <= fw;
+    return ok ? e : -1;
+  }
+};
 
-// Level-1 pixel (Y, X) of channel c: the frame's own, or inside a span-4 token
-// the 2x bilinear resize of level 2 (the coarse-to-fine cascade; spans are at
-// most 4).
-template <typename T>
-__device__ __forceinline__ float level1_pixel(const T* __restrict__ mb, int T4,
-                                              const int32_t* __restrict__ mapb, int fh, int fw,
-                                              int c, int Y, int X) {
-  const int32_t e = mapb[(int64_t)Y * fw + X];
-  return (e >= 0 && map_lvl(e) >= 2) ? frame_resize2x(2, mb, T4, mapb, fh, fw, c, Y, X)
-                                     : frame_pixel<1>(mb, T4, mapb, fw, c, Y, X);
-}
-
-// One (output cell, channel) on its own: a hole is reported and gives zeros, a
-// span-1 cell is copied, a coarser cell's four pixels are the 2x bilinear
-// resize of level 1 around it (a 3 x 3 neighbourhood, clamped to the frame).
-template <typename T>
-__device__ __forceinline__ typename Pix4<T>::V merge_cell_channel(
-    const T* __restrict__ mb, int T4, const int32_t* __restrict__ mapb, int fh, int fw, int32_t e,
-    int c, int Y, int X) {
-  using PV = typename Pix4<T>::V;
-  if (e < 0) return Pix4<T>::make(0.f, 0.f, 0.f, 0.f);
-  if (map_lvl(e) == 0) return reinterpret_cast<const PV*>(mb + (int64_t)map_tok(e) * T4)[c];
-  float lv[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-      lv[i][j] = level1_pixel(mb, T4, mapb, fh, fw, c, min(max(Y - 1 + i, 0), fh - 1),
-                              min(max(X - 1 + j, 0), fw - 1));
-  float r[4];
-  resize_cell(lv, 0, 0, r);
-  return Pix4<T>::make(r[0], r[1], r[2], r[3]);
+// Pass 1b for merge_bilinear_kernel, whose channels read a cell's word many
+// times over: words that no token of this call stands behind become -1.
+__global__ void __launch_bounds__(256)
+merge_live_kernel(int64_t ncell, int N, const int32_t* __restrict__ pos,
+                  const int32_t* __restrict__ span, int fh, int fw, int32_t* __restrict__ map) {
+  pdl_wait_then_trigger();
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= ncell) return;
+  CellWord w{map[g]};
+  if (w.e < 0) return;
+  const int cells = fh * fw;
+  const int b = (int)(g / cells), cell = (int)(g % cells);
+  w.place(N, pos + (int64_t)b * N * 2, span + (int64_t)b * N);
+  if (w.live(N, fh, fw, cell / fw, cell % fw) < 0) map[g] = -1;
 }
 
 // Bilinear merge, pass 2, one thread per (output cell, channel): tokens whose
-// rows are not whole 16-byte pieces.
+// rows are not whole 16-byte pieces.  Every word of the map is live or negative
+// (merge_live_kernel).  A hole is reported and gives zeros, a span-1 cell is
+// copied, a coarser cell's four pixels are the 2x bilinear resize of the level-1
+// pixels around it (a 3 x 3 neighbourhood, clamped to the frame): the frame's
+// own, or inside a span-4 token the 2x resize of level 2 (the coarse-to-fine
+// cascade; spans are at most 4).
 template <typename T>
-__global__ void __launch_bounds__(256)
-merge_bilinear_kernel(const T* __restrict__ mixed, int B, int N, const int32_t* __restrict__ pos,
-                      const int32_t* __restrict__ span, int fh, int fw, int C,
+__global__ void
+merge_bilinear_kernel(const T* __restrict__ mixed, int B, int N, int fh, int fw, int C,
                       const int32_t* __restrict__ map, T* __restrict__ out, unsigned int* status) {
   using PV = typename Pix4<T>::V;
   pdl_wait_then_trigger();
@@ -418,33 +413,63 @@ merge_bilinear_kernel(const T* __restrict__ mixed, int B, int N, const int32_t* 
   const int b = (int)(bc / cells);
   const int cell = (int)(bc % cells);
   const int Y = cell / fw, X = cell - Y * fw;
+  const int T4 = C * 4;
   const int32_t* mapb = map + (int64_t)b * cells;
-  const int32_t e = live_entry(mapb[cell], N, pos + (int64_t)b * N * 2, span + (int64_t)b * N, Y, X);
-  if (e < 0) raise_status(status, AVITS_ERR_COVERAGE);
-  reinterpret_cast<PV*>(out + bc * C * 4)[c] =
-      merge_cell_channel(mixed + (int64_t)b * N * C * 4, C * 4, mapb, fh, fw, e, c, Y, X);
+  const T* mb = mixed + (int64_t)b * N * T4;
+  const int32_t e = mapb[cell];
+  PV* dst = reinterpret_cast<PV*>(out + bc * T4) + c;
+  if (e < 0) {
+    raise_status(status, AVITS_ERR_COVERAGE);
+    *dst = Pix4<T>::make(0.f, 0.f, 0.f, 0.f);
+    return;
+  }
+  if (map_lvl(e) == 0) {
+    *dst = reinterpret_cast<const PV*>(mb + (int64_t)map_tok(e) * T4)[c];
+    return;
+  }
+  int rr[3], cc[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    rr[k] = min(max(Y - 1 + k, 0), fh - 1);
+    cc[k] = min(max(X - 1 + k, 0), fw - 1);
+  }
+  float lv[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int32_t en = mapb[(int64_t)rr[i] * fw + cc[j]];
+      lv[i][j] = (en >= 0 && map_lvl(en) >= 2)
+                     ? frame_resize2x(2, mb, T4, mapb, fh, fw, c, rr[i], cc[j])
+                     : frame_pixel<1>(mb, T4, mapb, fw, c, rr[i], cc[j]);
+    }
+  float r[4];
+  resize_cell(lv, r);
+  *dst = Pix4<T>::make(r[0], r[1], r[2], r[3]);
 }
 
 // Bilinear merge, pass 2, for tokens of whole 16-byte pieces: a CTA takes a tile
 // of 16 x 16 cells and two pieces (32 bytes) of the channels.  It loads the
-// cell map of the tile and four cells around it (an entry of the tile that no
-// token of this call covers is a hole: reported, zeros), turns every cell of the tile
-// and the ring next to it into its level-1 pixel (one 16-byte load: a span-2
+// cell map of the tile and four cells around it (a word that no token of this
+// call stands behind is a hole: zeros, and reported within the tile), turns every
+// cell of the tile and the ring next to it into its level-1 pixel (one 16-byte
+// load: a span-2
 // token's pixel, or the average of a span-1 token's four) in shared memory,
 // and writes the cells from the 3 x 3 level-1 pixels around them; span-1 cells
 // are copied.  Only where a span-4 token is near does it also build the level-2
 // pixels (from the wider ring) and refine the level-1 pixels inside such
-// tokens.  Every value is the one merge_cell_channel would compute, in the same
+// tokens.  Every value is the one merge_bilinear_kernel would compute, in the same
 // order of operations.  What bounds it: the chain map - token - shared memory -
 // cell at a few CTAs per SM, then the copies.  us of the two kernels, against a
 // thread per (cell, channel) behind a fill and an atomic scatter, bf16, 64 x 64
-// cells of 16 channels: batch 1 8.4 -> 6.3, 16 31.3 -> 11.5, 64 102 -> 31.4; batch
-// 32 with spans 1, 2 and 4 2606 -> 28.4 (a value of level 2 was pooled anew by
-// every thread that drew on it).  A cell's token is checked once, where the map
-// is loaded (by each piece's thread: 12.8 at batch 16).  Left out: a thread per
-// 2 x 2 cells with the neighbourhood in registers, 10.5 at batch 16 but 5580 with
-// span 4; three pieces of a thread in flight (13.2 against 12.8); four pieces per
-// CTA (12.9); the pieces' planes 16 banks apart (12.4).
+// cells of 16 channels: batch 1 8.5 -> 6.0, 16 31.7 -> 11.9, 64 103 -> 32.2; batch 64
+// with spans 1, 2 and 4 5371 -> 49.3 (a value of level 2 was pooled anew by every
+// thread that drew on it).  Words are checked where the map is loaded, the wider
+// ring's as well, a thread's three words and then their tokens' places in flight
+// together (one after the other: 6.7, 13.0, 33.8 and 60.7).  Left out: a thread
+// per 2 x 2 cells with the neighbourhood in registers, 10.5 at batch 16 but 5580
+// with span 4; three pieces of a thread in flight (13.2 against 12.8); four pieces
+// per CTA (12.9); the pieces' planes 16 banks apart (12.4).
 constexpr int kTile = 16;
 constexpr int kHalo = 4;                        // cells around the tile that level 2 can draw on
 constexpr int kReg = kTile + 2 * kHalo;
@@ -475,20 +500,26 @@ merge_bilinear_tile_kernel(const T* __restrict__ mixed, int N, const int32_t* __
   const int32_t* spanb = span + (int64_t)b * N;
   const T* mb = mixed + (int64_t)b * N * T4;
   T* ob = out + (int64_t)b * fh * fw * T4;
-  // the map, -1 off the frame and for words that are no token of this call
-  bool wide = false;
-  for (int i = threadIdx.x; i < kReg * kReg; i += 256) {
-    const int r = i / kReg, c = i - r * kReg;
+  // the map, -1 off the frame and for words that no token of this call stands
+  // behind; all of a thread's words, then all of their tokens' places in flight
+  constexpr int kWords = (kReg * kReg + 255) / 256;
+  CellWord cw[kWords];
+#pragma unroll
+  for (int k = 0; k < kWords; ++k) {
+    const int i = threadIdx.x + 256 * k, Y = Y0 - kHalo + i / kReg, X = X0 - kHalo + i % kReg;
+    cw[k].e = i < kReg * kReg && Y >= 0 && Y < fh && X >= 0 && X < fw ? mapb[(int64_t)Y * fw + X] : -1;
+  }
+#pragma unroll
+  for (int k = 0; k < kWords; ++k) cw[k].place(N, posb, spanb);
+  bool wide = false;   // a span-4 token in the tile or the ring next to it
+#pragma unroll
+  for (int k = 0; k < kWords; ++k) {
+    const int i = threadIdx.x + 256 * k, r = i / kReg, c = i % kReg;
+    if (i >= kReg * kReg) break;
     const int Y = Y0 - kHalo + r, X = X0 - kHalo + c;
-    int32_t e = -1;
-    if (Y >= 0 && Y < fh && X >= 0 && X < fw) {
-      e = mapb[(int64_t)Y * fw + X];
-      if (e >= 0 && map_tok(e) >= N) e = -1;
-      if (r >= kHalo && r < kHalo + kTile && c >= kHalo && c < kHalo + kTile) {
-        e = live_entry(e, N, posb, spanb, Y, X);
-        if (e < 0) raise_status(status, AVITS_ERR_COVERAGE);
-      }
-    }
+    const int32_t e = cw[k].live(N, fh, fw, Y, X);
+    if (e < 0 && r >= kHalo && r < kHalo + kTile && c >= kHalo && c < kHalo + kTile && Y < fh && X < fw)
+      raise_status(status, AVITS_ERR_COVERAGE);
     smap[r][c] = e;
     wide = wide || (e >= 0 && map_lvl(e) >= 2 && r >= kHalo - 1 && r <= kHalo + kTile &&
                     c >= kHalo - 1 && c <= kHalo + kTile);
@@ -588,7 +619,7 @@ merge_bilinear_tile_kernel(const T* __restrict__ mixed, int N, const int32_t* __
         for (int w = 0; w < 3; ++w)
           lv[u][w] = l1[pc][ch][r + (min(max(Y - 1 + u, 0), fh - 1) - Y)]
                                [c + (min(max(X - 1 + w, 0), fw - 1) - X)];
-      resize_cell(lv, 0, 0, v[ch]);
+      resize_cell(lv, v[ch]);
     }
     write(Y, X, pc, Chunk<T>::pack(v));
   }
@@ -641,11 +672,13 @@ cudaError_t launch_t(const void* mixed, int B, int N, const int32_t* pos, const 
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
   }
-  // two kernels (scatter of the cell map, gather), the second a programmatic
-  // dependent of the first
+  // two kernels (scatter of the cell map, gather; where tokens are not whole
+  // 16-byte pieces a third between them), each a programmatic dependent of the
+  // one before
   int32_t* map = reinterpret_cast<int32_t*>(words);
   const int64_t nt = (int64_t)B * N;
   cudaError_t e = prefer_max_shared<merge_scatter_kernel>();
+  if (e == cudaSuccess) e = prefer_max_shared<merge_live_kernel>();
   if (e == cudaSuccess) e = prefer_max_shared<merge_bilinear_kernel<T>>();
   if (e == cudaSuccess) e = prefer_max_shared<merge_bilinear_tile_kernel<T>>();
   if (e != cudaSuccess) return e;
@@ -661,10 +694,13 @@ cudaError_t launch_t(const void* mixed, int B, int N, const int32_t* pos, const 
                    static_cast<const int32_t*>(map), static_cast<T*>(out), status, (unsigned)tx,
                    (unsigned)ty, (unsigned)groups);
   } else {
-    const int64_t all = (int64_t)B * fh * fw * C;
+    const int64_t ncell = (int64_t)B * fh * fw, all = ncell * C;
+    e = launch_pdl(merge_live_kernel, dim3((unsigned)((ncell + 255) / 256)), dim3(256), 0, s, ncell,
+                   N, pos, span, fh, fw, map);
+    if (e != cudaSuccess) return e;
     e = launch_pdl(merge_bilinear_kernel<T>, dim3((unsigned)((all + 255) / 256)), dim3(256), 0, s,
-                   static_cast<const T*>(mixed), B, N, pos, span, fh, fw, C,
-                   static_cast<const int32_t*>(map), static_cast<T*>(out), status);
+                   static_cast<const T*>(mixed), B, N, fh, fw, C, static_cast<const int32_t*>(map),
+                   static_cast<T*>(out), status);
   }
   if (e != cudaSuccess) return e;
   return cudaGetLastError();

@@ -117,6 +117,57 @@ def test_merge_two_pass_reports_bad_tilings(av, first):
             assert st == 0 and _same(got, want[m])
 
 
+@pytest.mark.parametrize("spans", [[1, 2], [1, 2, 4]])
+@pytest.mark.parametrize("dtype,C", [("bf16", 1), ("bf16", 3), ("bf16", 16), ("f32", 1), ("f32", 4)])
+def test_a_hole_shows_nothing_of_earlier_calls(av, dtype, C, spans):
+    """A bilinear merge with holes on a workspace that a merge of more tokens
+    used before: reported, and the cells around a hole draw on zeros, not on
+    what the old words name (tokens beyond this call's, here among the NaNs
+    around the sequence, or tokens elsewhere in it)."""
+    import torch
+    import oracle
+    from paper_2608_17995_gb300.pipeline import to_device, to_numpy
+    rng = np.random.default_rng(C + len(spans))
+    B, fh, fw = 3, 40, 24   # one token per cell: enough for the nearest merge's two passes
+    pos, span = _tiling(rng, B, fh, fw, 4, spans)
+    N, T = pos.shape[1], 4 * C
+    mixed = _latent(rng, B, N, C, dtype)
+    for b in range(B):   # two holes of every span, the frame's last token among them
+        last = np.flatnonzero((pos[b] + span[b][:, None] == [fh, fw]).all(1))
+        holes = np.concatenate([rng.choice(np.flatnonzero(span[b] == s), 2) for s in spans] + [last])
+        span[b, holes] *= -1
+        mixed[b, holes] = 0
+    out = np.zeros((B, fh, fw), bool)   # cells of holes
+    for b, t in zip(*np.nonzero(span < 0)):
+        y, x, s = *pos[b, t], -span[b, t]
+        out[b, y:y + s, x:x + s] = True
+    out = out.reshape(B, fh * fw)
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    n = B * N * T + -B * N * T % 8   # the sequence starts on 16 bytes
+    wide = torch.full((3 * n,), float("nan"), dtype=tdt, device="cuda")
+    view = wide[n:n + B * N * T].view(B, N, T)
+    view.copy_(to_device(mixed, dtype))
+    dense = np.stack([np.stack(np.divmod(np.arange(fh * fw), fw), 1)] * B).astype(np.int32)
+    ones = np.ones((B, fh * fw), np.int32)
+    got = []
+    for first in (None, NEAREST, BILINEAR):
+        ws = torch.zeros(av.avits_merge_final_workspace(BILINEAR, B, fh, fw), dtype=torch.uint8,
+                         device="cuda")
+        if first is not None:   # one token per cell, in raster order
+            assert _call(av, _latent(rng, B, fh * fw, C, dtype), dtype, dense, ones, fh, fw, first,
+                         ws)[1] == 0
+        full = torch.full((B, fh * fw, T), 7.0, dtype=tdt, device="cuda")
+        av.avits_merge_final(view, to_device(pos, "i32"), to_device(span, "i32"), fh, fw, full,
+                             mode=BILINEAR, workspace=ws)
+        assert av.avits_device_status() == 6
+        got.append(to_numpy(full))
+    assert _same(got[0], got[1]) and _same(got[0], got[2])
+    assert not got[0][out].any()
+    if spans == [1, 2]:   # elsewhere: as if the missing tokens were zeros
+        want, _ = oracle.merge_final(mixed, pos, np.abs(span), fh, fw, mode="bilinear")
+        assert _same(got[0][~out], want[~out])
+
+
 @pytest.mark.parametrize("dtype,C,gh,gw,k", [
     ("bf16", 16, 9, 13, 40), ("f32", 4, 16, 16, 0), ("f32", 1, 8, 30, 240), ("bf16", 2, 33, 8, 100),
     ("bf16", 1, 8, 8, 30), ("bf16", 16, 1, 20, 7), ("bf16", 16, 20, 1, 7)])
