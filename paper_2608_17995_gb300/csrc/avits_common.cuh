@@ -111,8 +111,10 @@ __device__ __forceinline__ void pdl_wait_then_trigger() {
 // All kernels of the path prefer the same (all shared) L1/shared carveout:
 // two kernels with different carveouts cannot share an SM, which would stop
 // a programmatic dependent from starting beside its predecessor.  Set once
-// per kernel and device.
-template <auto Kernel>
+// per kernel and device, with the opt-in to kDynamic bytes of dynamic shared
+// memory where the sizes of some call ask for more than 48 KB less the kernel's
+// static arrays.
+template <auto Kernel, int kDynamic = 0>
 inline cudaError_t prefer_max_shared() {
   static int done[64] = {};
   int dev = 0;
@@ -121,6 +123,8 @@ inline cudaError_t prefer_max_shared() {
   if (dev >= 0 && dev < 64 && __atomic_load_n(&done[dev], __ATOMIC_ACQUIRE)) return cudaSuccess;
   e = cudaFuncSetAttribute(Kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                            cudaSharedmemCarveoutMaxShared);
+  if (kDynamic > 0 && e == cudaSuccess)
+    e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynamic);
   if (e == cudaSuccess && dev >= 0 && dev < 64) __atomic_store_n(&done[dev], 1, __ATOMIC_RELEASE);
   return e;
 }

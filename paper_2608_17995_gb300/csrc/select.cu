@@ -589,23 +589,6 @@ cudaError_t launch_fuse_select(const float* A, const float* V, const float* pert
                                uint8_t* mask, int32_t* tok_offset, unsigned int* status,
                                cudaStream_t s) {
   const size_t smem = (size_t)M * sizeof(uint32_t);
-  if (smem > 48 * 1024) {
-    // opt in once per device to the largest size any call can ask for
-    static int done[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (!(dev >= 0 && dev < 64 && __atomic_load_n(&done[dev], __ATOMIC_ACQUIRE))) {
-      const int mx = (int)(kSelectMaxM * sizeof(uint32_t));
-      e = cudaFuncSetAttribute(fuse_select_kernel<kMaxThreads, 0>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      if (e != cudaSuccess) return e;
-      e = cudaFuncSetAttribute(fuse_select_kernel<kMaxThreads, kMaxRegKeys>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-      if (e != cudaSuccess) return e;
-      if (dev >= 0 && dev < 64) __atomic_store_n(&done[dev], 1, __ATOMIC_RELEASE);
-    }
-  }
   // 256 threads up to M = 256, 512 beyond (up to 2 keys per thread at
   // FLUX-1024: the per-key work of the fuse step is the longest part, measured
   // 3.50 -> 3.33 us against 256 threads); shared memory only above 4096
@@ -629,7 +612,8 @@ cudaError_t launch_fuse_select(const float* A, const float* V, const float* pert
   if (ce == cudaSuccess) ce = prefer_max_shared<fuse_select_kernel<kMaxThreads, 2>>();
   if (ce == cudaSuccess) ce = prefer_max_shared<fuse_select_kernel<kMaxThreads, 4>>();
   if (ce == cudaSuccess) ce = prefer_max_shared<fuse_select_kernel<kMaxThreads, kMaxRegKeys>>();
-  if (ce == cudaSuccess) ce = prefer_max_shared<fuse_select_kernel<kMaxThreads, 0>>();
+  if (ce == cudaSuccess)
+    ce = prefer_max_shared<fuse_select_kernel<kMaxThreads, 0>, kSelectMaxM * (int)sizeof(uint32_t)>();
   if (ce != cudaSuccess) return ce;
   const SelArgs g{A, V, perturb, M, alpha, eps, k, S, sel_idx, mask, tok_offset, status};
   cudaError_t e = launch_pdl(kern, dim3(B), dim3(threads), smem, s, g);
@@ -642,6 +626,7 @@ namespace {
 constexpr int kFusedThreads = 512;
 constexpr int kFusedCtasTotal = 152;   // CTAs of the fused kernel over all elements
 constexpr int kFusedMaxM = kFusedThreads * kMaxRegKeys;   // 4096
+constexpr int kFusedSmem = 96 * 1024;   // the most that scores and staged rows take
 
 template <typename T, bool kBilinear>
 cudaError_t launch_fused_t(const SelArgs& g, const UpsampleArgs<T>& u, int B, int M,
@@ -651,10 +636,13 @@ cudaError_t launch_fused_t(const SelArgs& g, const UpsampleArgs<T>& u, int B, in
               : per <= 2 ? select_upsample_kernel<kFusedThreads, 2, T, kBilinear>
               : per <= 4 ? select_upsample_kernel<kFusedThreads, 4, T, kBilinear>
                          : select_upsample_kernel<kFusedThreads, 8, T, kBilinear>;
-  cudaError_t e = prefer_max_shared<select_upsample_kernel<kFusedThreads, 1, T, kBilinear>>();
-  if (e == cudaSuccess) e = prefer_max_shared<select_upsample_kernel<kFusedThreads, 2, T, kBilinear>>();
-  if (e == cudaSuccess) e = prefer_max_shared<select_upsample_kernel<kFusedThreads, 4, T, kBilinear>>();
-  if (e == cudaSuccess) e = prefer_max_shared<select_upsample_kernel<kFusedThreads, 8, T, kBilinear>>();
+  cudaError_t e = prefer_max_shared<select_upsample_kernel<kFusedThreads, 1, T, kBilinear>, kFusedSmem>();
+  if (e == cudaSuccess)
+    e = prefer_max_shared<select_upsample_kernel<kFusedThreads, 2, T, kBilinear>, kFusedSmem>();
+  if (e == cudaSuccess)
+    e = prefer_max_shared<select_upsample_kernel<kFusedThreads, 4, T, kBilinear>, kFusedSmem>();
+  if (e == cudaSuccess)
+    e = prefer_max_shared<select_upsample_kernel<kFusedThreads, 8, T, kBilinear>, kFusedSmem>();
   if (e != cudaSuccess) return e;
   // about 2 tokens per warp, at most one CTA per SM over all elements (every
   // CTA repeats its element's selection)
@@ -667,14 +655,9 @@ cudaError_t launch_fused_t(const SelArgs& g, const UpsampleArgs<T>& u, int B, in
   int stage_rows = std::min(M, chunk + 2 * halo);
   const size_t head = ((9 * (size_t)M + 15) / 16) * 16;
   if (row_bytes % 16 != 0 || (reinterpret_cast<uintptr_t>(u.latent) & 15u) != 0 ||
-      head + stage_rows * row_bytes > 96 * 1024)
+      head + stage_rows * row_bytes > kFusedSmem)
     stage_rows = 0;
   const size_t smem = head + (size_t)stage_rows * row_bytes;
-  // the 48 KB that need no opt-in hold the kernel's static arrays as well
-  if (smem > 40 * 1024) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    if (e != cudaSuccess) return e;
-  }
   e = launch_pdl(kern, dim3((unsigned)(B * parts)), dim3(kFusedThreads), smem, s, g, u, parts,
                  stage_rows);
   if (e != cudaSuccess) return e;
