@@ -12,14 +12,13 @@
 //
 // avits_score_temporal_var: Eq. 6-7, unbiased variance over N_T snapshots
 // averaged over channels; two passes over the snapshot values held in
-// registers (mean, then squared deviations).  Main path: one CTA per token,
-// 16-byte loads, the N_T vectors of a position all issued before they are
-// reduced (HBM-bound: N_T * D * elt bytes per token).
+// registers (mean, then squared deviations).  Main path: a CTA, a warp or part
+// of one per token, 16-byte loads, the N_T vectors of a position all issued
+// before they are reduced (HBM-bound: N_T * D * elt bytes per token).
 #include "avits_common.cuh"
 #include "avits_internal.h"
 
 #include <algorithm>
-#include <cmath>
 
 namespace avits {
 namespace {
@@ -320,8 +319,12 @@ __device__ __forceinline__ float vec_elem<__nv_bfloat16>(const uint4& v, int e) 
 // threads are without a vector and no token waits at a barrier.  With a CTA
 // per token throughout, us before -> now: D = 128 bf16, 2 snapshots, 65536
 // tokens 59.6 -> 12.4, 16384 tokens 13.6 -> 4.0; D = 768, 3 snapshots, 16384
-// tokens 21.0 -> 15.2 (1024 tokens 2.8 -> 2.9); D = 128 fp32, 4 snapshots,
-// 16384 tokens 16.0 -> 7.4.
+// tokens 21.0 -> 15.2; D = 128 fp32, 4 snapshots, 16384 tokens 16.0 -> 7.4.
+// Rows of 33 to 127 vectors keep a CTA per token while the tokens are few: a
+// warp's two to four rounds of loads are then the longest chain.  (A lane adds
+// its vectors up in one chain, a CTA its four warps' sums at the end, so the two
+// differ in the last bits; a warp that sums each 32 vectors on their own gives the
+// CTA's bits and costs 7 % at 16384 tokens.)
 constexpr int kVarThreads = 128;
 
 template <typename T, int kNT, int kLanes>
@@ -389,9 +392,19 @@ temporal_var_vec_kernel(SnapPtrs snaps, int n_t, int64_t ntok, int D, float* __r
 }
 
 template <typename T, int kNT>
-void launch_var_lanes(const SnapPtrs& sp, int n_t, int64_t ntok, int D, float* V, cudaStream_t s) {
+void launch_var_lanes(const SnapPtrs& sp, int n_t, int64_t ntok, int D, float* V, int num_sms,
+                      cudaStream_t s) {
   const int nv = D * (int)sizeof(T) / 16;
-  const int lanes = nv <= 8 ? 8 : nv <= 16 ? 16 : nv < kVarThreads ? 32 : kVarThreads;
+  // Few tokens: while the CTAs are about one wave; longer where a warp's rounds
+  // hold many registers each.  us with a CTA / a warp per token, bf16: D = 264, 3
+  // snapshots, 300 tokens 2.3 / 2.5, 1500 3.1 / 2.9; D = 768, 3 snapshots, 300
+  // 2.4 / 2.9, 1500 3.35 / 3.5, 2048 3.9 / 3.75; D = 1000, 6 snapshots, 300 3.1 /
+  // 4.6, 2048 7.6 / 8.8, 4096 13.2 / 14.1, 6000 18.9 / 18.7.
+  const int per_sm = nv * n_t > 600 ? 28 : nv > 64 ? 12 : 8;
+  const bool few = ntok <= (int64_t)num_sms * per_sm;
+  const int lanes = nv <= 8    ? 8
+                    : nv <= 16 ? 16
+                    : nv <= 32 || (nv < kVarThreads && !few) ? 32 : kVarThreads;
   // a plain launch: as a programmatic dependent the waiting CTAs took SM slots
   // from the kernel before and measured slower (grid-stride beyond 2^31 - 1)
   const int per = kVarThreads / lanes;
@@ -404,10 +417,11 @@ void launch_var_lanes(const SnapPtrs& sp, int n_t, int64_t ntok, int D, float* V
 }
 
 template <typename T>
-void launch_var_vec(const SnapPtrs& sp, int n_t, int64_t ntok, int D, float* V, cudaStream_t s) {
-  if (n_t <= 4) launch_var_lanes<T, 4>(sp, n_t, ntok, D, V, s);
-  else if (n_t <= 8) launch_var_lanes<T, 8>(sp, n_t, ntok, D, V, s);
-  else launch_var_lanes<T, kMaxSnapshots>(sp, n_t, ntok, D, V, s);
+void launch_var_vec(const SnapPtrs& sp, int n_t, int64_t ntok, int D, float* V, int num_sms,
+                    cudaStream_t s) {
+  if (n_t <= 4) launch_var_lanes<T, 4>(sp, n_t, ntok, D, V, num_sms, s);
+  else if (n_t <= 8) launch_var_lanes<T, 8>(sp, n_t, ntok, D, V, num_sms, s);
+  else launch_var_lanes<T, kMaxSnapshots>(sp, n_t, ntok, D, V, num_sms, s);
 }
 
 }  // namespace
@@ -544,8 +558,8 @@ cudaError_t launch_temporal_var(const void* const* snaps, int n_t, avits_dtype d
   bool vec = ((int64_t)D * elt) % 16 == 0;
   for (int i = 0; i < n_t; ++i) vec = vec && (reinterpret_cast<uintptr_t>(snaps[i]) & 15u) == 0;
   if (vec) {
-    if (dt == AVITS_BF16) launch_var_vec<__nv_bfloat16>(sp, n_t, ntok, D, V, s);
-    else launch_var_vec<float>(sp, n_t, ntok, D, V, s);
+    if (dt == AVITS_BF16) launch_var_vec<__nv_bfloat16>(sp, n_t, ntok, D, V, num_sms, s);
+    else launch_var_vec<float>(sp, n_t, ntok, D, V, num_sms, s);
     return cudaGetLastError();
   }
   const int grid = grid_for(ntok, num_sms);

@@ -44,6 +44,31 @@ def test_variance_row_widths(av, dtype, vectors, n_t, N):
     np.testing.assert_allclose(to_numpy(V), oracle.score_temporal_var(snaps), rtol=1e-5, atol=1e-7)
 
 
+@pytest.mark.parametrize("dtype,vectors", [("bf16", 1), ("bf16", 16), ("bf16", 33), ("bf16", 96),
+                                           ("f32", 127), ("bf16", 127), ("bf16", 128)])
+@pytest.mark.parametrize("n_t", [2, 3, 6, 16])
+def test_variance_many_tokens(av, dtype, vectors, n_t):
+    """More tokens than the widest of the rules for few, and a few of them alone,
+    against the oracle.  The two sum a row's 16-byte vectors in another order for
+    33 to 127 of them and in the same one for all other widths."""
+    import torch
+    import oracle
+    from paper_2608_17995_gb300.pipeline import to_numpy
+    D, N = vectors * (4 if dtype == "f32" else 8), 4500
+    g = torch.Generator(device="cuda").manual_seed(D + n_t)
+    snaps = [torch.randn(1, N, D, generator=g, device="cuda").to(
+        torch.bfloat16 if dtype == "bf16" else torch.float32) for _ in range(n_t)]
+    V, few = torch.full((1, N), float("nan"), device="cuda"), torch.full((1, 70), float("nan"), device="cuda")
+    av.avits_score_temporal_var(snaps, V)
+    av.avits_score_temporal_var([s[:, -70:].contiguous() for s in snaps], few)
+    assert av.avits_device_status() == 0
+    if not 32 < vectors < 128:
+        assert torch.equal(V[:, -70:], few)
+    want = oracle.score_temporal_var([to_numpy(s) for s in snaps])
+    np.testing.assert_allclose(to_numpy(V), want, rtol=1e-5, atol=1e-7)
+    np.testing.assert_allclose(to_numpy(few), want[:, -70:], rtol=1e-5, atol=1e-7)
+
+
 @pytest.mark.parametrize("dtype,B,H,M,L,D", [
     ("bf16", 1, 1, 130, 20, 8),        # 64 rows of 16 bytes per copy, a ragged last one
     ("bf16", 3, 2, 257, 40, 128),
