@@ -142,7 +142,9 @@ temporal_scalar_kernel(const T* __restrict__ ht, const T* __restrict__ hp, int64
 // SM with the spatial kernel's CTA, so the two can run concurrently.  Beside a
 // running kernel, where one CTA per SM has the work of all, narrower rows fill
 // the same 24 KB (a token per warp and more; D = 64: 19.7 -> 13.7 us for both
-// scores of 8 x 12 heads x 500 tokens).
+// scores of 8 x 12 heads x 500 tokens), as far as every SM still has some (144
+// tokens of D = 128 in 3 CTAs of 48: 7.1 us for both scores of 2 heads, in 72 of
+// 2: 6.0).
 constexpr int kStageTokens = 2;
 constexpr int kOverlapBytes = 24 * 1024;
 constexpr int kOverlapMaxTokens = 64;
@@ -432,8 +434,11 @@ cudaError_t launch_staged(const void* ht, const void* hp, int64_t ntok, int D, f
                           int num_sms, unsigned int* status, cudaStream_t s, float beside_us = 0.f) {
   const size_t row = (size_t)D * sizeof(T);
   int tpc = (int)std::min<size_t>(kStageTokens, kStageBytesMax / (2 * row));
-  if (kOverlapped)
-    tpc = std::max(tpc, (int)std::min<size_t>(kOverlapMaxTokens, kOverlapBytes / (2 * row)));
+  if (kOverlapped) {
+    const int64_t per_sm = (ntok + std::max(num_sms, 1) - 1) / std::max(num_sms, 1);
+    const int64_t fit = std::min<int64_t>(kOverlapMaxTokens, (int64_t)(kOverlapBytes / (2 * row)));
+    tpc = std::max(tpc, (int)std::min(fit, per_sm));
+  }
   const size_t smem = 2 * (size_t)tpc * row;
   static int done[64] = {};
   int dev = 0;

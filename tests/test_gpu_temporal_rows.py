@@ -70,7 +70,9 @@ def test_variance_many_tokens(av, dtype, vectors, n_t):
 
 
 @pytest.mark.parametrize("dtype,B,H,M,L,D", [
-    ("bf16", 1, 1, 130, 20, 8),        # 64 rows of 16 bytes per copy, a ragged last one
+    ("bf16", 1, 1, 130, 20, 8),        # fewer rows than SMs: two per copy
+    ("bf16", 1, 1, 12000, 20, 8),      # 64 rows of 16 bytes per copy, a ragged last one
+    ("bf16", 1, 1, 1000, 20, 128),     # seven rows per copy
     ("bf16", 3, 2, 257, 40, 128),
     ("bf16", 2, 1, 4000, 24, 3072),    # several rounds beside a short spatial kernel
     ("bf16", 1, 1, 900, 16, 8192),     # one row per copy
