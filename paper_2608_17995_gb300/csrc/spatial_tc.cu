@@ -59,10 +59,10 @@
 //                 buffer; one TMEM lane (= one query row) per thread, 32
 //                 columns per tcgen05.ld, ex2 on the MUFU against the running
 //                 row maximum with packed f32x2 FMA/add.  The exact maximum of
-//                 the 32 is only computed when their sum would leave [0, 2^64)
-//                 (first keys, a larger logit, NaN).  32 at a time, load and
-//                 wait in one statement: 89.1 -> 84.0 us; 16 with the next 16
-//                 loading 89.1, 64 at a time 102.  The text keys
+//                 the 32 is only computed for a row's first keys and when their
+//                 sum would leave [0, 2^64) (a larger logit, NaN).  32 at a time,
+//                 load and wait in one statement: 89.1 -> 84.0 us; 16 with the
+//                 next 16 loading 89.1, 64 at a time 102.  The text keys
 //                 come first, so the text sum is a prefix of the row sum.  At
 //                 d = 128 a 128x128 tile costs the tensor pipe and the MUFU
 //                 (32 ex2 / clock / SM) the same 512 cycles; evaluating part
@@ -161,35 +161,42 @@ __device__ __forceinline__ void merge_stat(RowStat& a, float m2, float la2, floa
 
 // 32 keys that are all valid and all text (kText) or all image keys: the
 // common case, kept free of the masking and boundary logic (a branch on the
-// key kind per 16 keys measured ~15% slower on the whole item).
+// key kind per 16 keys measured ~15% slower on the whole item).  `first`
+// (uniform): the row's first keys, whose maximum is always needed: sums against
+// no maximum thrown away and a chain of 32 additions in their place made calls of
+// one or two items per CTA slower (24 heads x 256 x 768: 7.7 us, now 7.3; with 16
+// columns at a time 7.3; 1024 x 1536 13.1 -> 12.6).
 template <bool kText>
-__device__ __forceinline__ void process_cols_full(const uint32_t (&v)[32], float c, RowStat& st) {
-  const float nm = -st.m;
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+__device__ __forceinline__ void process_cols_full(const uint32_t (&v)[32], float c, bool first,
+                                                  RowStat& st) {
+  const auto sum = [&](float nm) {   // of 2^(c v + nm)
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll
-  for (int e = 0; e < 32; e += 4) {
-    float x0, x1, x2, x3;
-    ffma2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), c, nm, x0, x1);
-    ffma2(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]), c, nm, x2, x3);
-    fadd2(s0, s1, ex2(x0), ex2(x1));
-    fadd2(s2, s3, ex2(x2), ex2(x3));
-  }
-  fadd2(s0, s1, s2, s3);
-  float cs = s0 + s1;
+    for (int e = 0; e < 32; e += 4) {
+      float x0, x1, x2, x3;
+      ffma2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), c, nm, x0, x1);
+      ffma2(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]), c, nm, x2, x3);
+      fadd2(s0, s1, ex2(x0), ex2(x1));
+      fadd2(s2, s3, ex2(x2), ex2(x3));
+    }
+    fadd2(s0, s1, s2, s3);
+    return s0 + s1;
+  };
+  float cs = INFINITY;
+  if (!first) cs = sum(-st.m);
   if (!(cs < 0x1p64f)) {
     // first keys of a row, a logit 64 log2-units above the running maximum,
     // or a NaN: take the exact maximum and rescale the running sums
-    float cm = __uint_as_float(v[0]);
+    float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-    for (int e = 1; e < 32; ++e) cm = fmaxf(cm, __uint_as_float(v[e]));
-    const float mx = fmaxf(st.m, cm * c);
+    for (int e = 0; e < 32; e += 2)
+      m[(e >> 1) & 3] = max3(m[(e >> 1) & 3], __uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+    const float mx = fmaxf(st.m, fmaxf(max3(m[0], m[1], m[2]), m[3]) * c);
     const float corr = ex2(st.m - mx);
     st.la *= corr;
     st.lt *= corr;
     st.m = mx;
-    cs = 0.f;
-#pragma unroll
-    for (int e = 0; e < 32; ++e) cs += ex2(fmaf(__uint_as_float(v[e]), c, -mx));
+    cs = sum(-mx);
   }
   st.la += cs;
   if (kText) st.lt += cs;
@@ -350,12 +357,12 @@ __device__ __forceinline__ void process_chunk_masked(const uint32_t (&r)[16], in
 
 template <int kKind>
 __device__ __forceinline__ void softmax_item(uint32_t tb, int c0, int Nk, int L, float c,
-                                             RowStat& st, uint64_t* s_empty, int lane,
+                                             RowStat& st, uint64_t* s_empty, int lane, bool first,
                                              uint32_t w0 = 0u, uint32_t w1 = 0u) {
   uint32_t v[32];
   auto cols = [&](int k) {   // columns 32 k .. 32 k + 31 of the warp's 64
     if constexpr (kKind == kItemText || kKind == kItemImage) {
-      process_cols_full<kKind == kItemText>(v, c, st);
+      process_cols_full<kKind == kItemText>(v, c, first && k == 0, st);
     } else {
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
@@ -694,17 +701,17 @@ spatial_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             const uint32_t w1 = __ballot_sync(0xffffffffu, mb1);
             const bool full = c0 + 64 <= p.Nk;
             if (full && (w0 & w1) == 0xffffffffu)
-              softmax_item<kItemText>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane);
+              softmax_item<kItemText>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane, j == 0);
             else if (full && (w0 | w1) == 0u)
-              softmax_item<kItemImage>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane);
+              softmax_item<kItemImage>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane, j == 0);
             else
-              softmax_item<kItemMasked>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane, w0, w1);
+              softmax_item<kItemMasked>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane, j == 0, w0, w1);
           } else if (c0 + 64 <= p.Nk && c0 + 64 <= p.L)
-            softmax_item<kItemText>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane);
+            softmax_item<kItemText>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane, j == 0);
           else if (c0 + 64 <= p.Nk && c0 >= p.L)
-            softmax_item<kItemImage>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane);
+            softmax_item<kItemImage>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane, j == 0);
           else
-            softmax_item<kItemGeneral>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane);
+            softmax_item<kItemGeneral>(tb, c0, p.Nk, p.L, p.c_log2, st, empty, lane, j == 0);
         } else {
           __syncwarp();
           if (lane == 0) mbar_arrive(&bars->s_empty[t][sb]);
