@@ -12,8 +12,9 @@
 //                for a mixed input, from level log2(s) of the input frame's
 //                pixel pyramid through its cell map (frame_map.cuh).
 // Token rows of whole 16-byte chunks: each lane writes chunks (coalesced);
-// otherwise, and for the pixel pyramid of a mixed input, lanes split the
-// (child, channel) work, each writing the 4 pixels of one channel of one child.
+// otherwise, for the pixel pyramid of a mixed input, and for bilinear children of
+// up to 8 bf16 channels, lanes split the (child, channel) work, each writing the 4
+// pixels of one channel of one child.
 // Lanes 0-3 write the position / span / source maps.
 #pragma once
 
@@ -67,7 +68,10 @@ struct SharedRows {
 // Bound by instructions and the latency of a token's chain (a warp per token),
 // not by bytes; a lane per (child, channel) read nine scalars for each.  One
 // launch with the selection, 32 x 32 grids of 16 bf16 channels, us: batch 1 5.6 ->
-// 5.2, 16 13.5 -> 11.5, 64 34.4 -> 29.5.
+// 5.2, 16 13.5 -> 11.5, 64 34.4 -> 29.5.  Up to 8 bf16 channels the lanes hold every
+// (child, channel) in one round and half of them would be without a piece of two
+// channels: 8 channels 11.4 (10.3 by channels) at batch 16, 4 channels 30.3 (26.1) at
+// 64; 12 channels 11.5 (13.4) and 30.5 (35.5).
 template <typename T, typename Src>
 __device__ __forceinline__ uint4 bilinear_child(const Src& rows, int b_elem, int gh, int gw, int y,
                                                 int x, int a, int b, int j) {
@@ -147,7 +151,8 @@ __device__ __forceinline__ void upsample_token(const UpsampleArgs<T>& u, const S
   const T* src = rows.row(b, i);
   const int64_t out_tok0 = (int64_t)b * u.n_out + o;
   const int tb = T4 * (int)sizeof(T);
-  if ((tb & 15) == 0 && (!kBilinear || !sel || !u.map)) {
+  const bool pieces = Chunk<T>::kCh == 1 || 4 * C > 32;   // of bilinear children
+  if ((tb & 15) == 0 && (!kBilinear || !sel || (pieces && !u.map))) {
     // 16-byte chunks: a deferred token is copied; nearest gives each child
     // (a, b) of a selected one the chunk whose channel pixels all equal the
     // parent's pixel (a, b), bilinear on a dense grid resizes around it; one

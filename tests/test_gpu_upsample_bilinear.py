@@ -7,7 +7,8 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dtype,C", [("bf16", 2), ("bf16", 3), ("bf16", 16), ("f32", 1), ("f32", 5)])
+@pytest.mark.parametrize("dtype,C", [("bf16", 2), ("bf16", 3), ("bf16", 8), ("bf16", 10),
+                                     ("bf16", 16), ("f32", 1), ("f32", 5)])
 @pytest.mark.parametrize("gh,gw", [(1, 1), (1, 7), (6, 1), (2, 2), (9, 17), (8, 33)])
 def test_bilinear_pieces(gh, gw, dtype, C):
     import torch
