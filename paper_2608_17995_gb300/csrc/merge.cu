@@ -3,8 +3,8 @@
 // spatial order).
 //
 // Nearest: full-res pixel (Y,X) of a token at (y,x) with span s takes token
-// pixel ((Y-2y)/s, (X-2x)/s).  Few tokens (a batch of one): one warp per token
-// writes its s x s cells in one pass; every cell is claimed by an atomicExch of
+// pixel ((Y-2y)/s, (X-2x)/s).  Few tokens (a batch of one): a warp, or 8 lanes, per
+// token write its s x s cells in one pass; every cell is claimed by an atomicExch of
 // this call's tag into a claim map in the caller's workspace (an old value equal
 // to the tag = a cell covered twice).  More tokens: pass 1 writes each token's
 // index into the words of its cells with plain stores, pass 2 goes over the
@@ -60,26 +60,28 @@ __device__ __forceinline__ void count_cells(MergeHeader* hdr, unsigned long long
   hdr->count = 0ull;
 }
 
-// Few tokens: one warp per token, one pass.  A token's area is known once its position and
+// Few tokens: kLanes lanes (a warp, or part of one) per token, one pass.  A token's area is known once its position and
 // span are read, so the CTA's count goes out first; the claims, the count's
 // atomic and the pixel loads are then in flight together and their results
 // are examined last: the check adds no round trip to the copy's two
 // (position, then pixels).
-template <typename T>
+template <typename T, int kLanes>
 __global__ void __launch_bounds__(8 * 32)
 merge_nearest_warp_kernel(const T* __restrict__ mixed, int B, int N,
                           const int32_t* __restrict__ pos, const int32_t* __restrict__ span,
                           int fh, int fw, int C, T* __restrict__ out, MergeHeader* hdr,
                           uint32_t* __restrict__ claim, unsigned int* status) {
   using PV = typename Pix4<T>::V;
-  constexpr int kStage = 1024;   // a token of up to 1 KB takes the vector path
+  constexpr int kToks = 8 * 32 / kLanes;   // per CTA
+  constexpr int kStage = 8192 / kToks;     // a token of up to so many bytes takes the vector path
   pdl_wait_then_trigger();
-  __shared__ __align__(16) uint8_t stage_all[8 * kStage];
+  __shared__ __align__(16) uint8_t stage_all[kToks * kStage];
   __shared__ unsigned int cta_cells;
   if (threadIdx.x == 0) cta_cells = 0u;
   const uint32_t last = *reinterpret_cast<volatile uint32_t*>(&hdr->last_tag);
-  const int lane = threadIdx.x & 31;
-  const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x % kLanes, slot = threadIdx.x / kLanes;
+  const unsigned group = (0xffffffffu >> (32 - kLanes)) << (threadIdx.x & 31 & ~(kLanes - 1));
+  const int64_t t = (int64_t)blockIdx.x * kToks + slot;
   int b = 0, y = 0, x = 0, sp = 0;
   bool valid = false;
   if (t < (int64_t)B * N) {
@@ -98,7 +100,7 @@ merge_nearest_warp_kernel(const T* __restrict__ mixed, int B, int N,
     v = atomicAdd(&hdr->count, (1ull << 40) | (unsigned long long)cta_cells) +
         ((1ull << 40) | (unsigned long long)cta_cells);
   const uint32_t tag = next_tag(last);
-  uint32_t old0 = 0u, old1 = 0u;   // claims of cells lane and lane + 32
+  uint32_t old0 = 0u, old1 = 0u;   // claims of cells lane and lane + kLanes
   bool twice = false;
   if (valid) {
     const int64_t base = (int64_t)b * fh * fw;
@@ -107,21 +109,21 @@ merge_nearest_warp_kernel(const T* __restrict__ mixed, int B, int N,
     const T* src = mixed + t * T4;
     const int tb = T4 * (int)sizeof(T);
     const bool vec = (tb & 15) == 0 && tb <= kStage;
-    uint8_t* stage = stage_all + (threadIdx.x >> 5) * kStage;
+    uint8_t* stage = stage_all + slot * kStage;
     if (vec)
-      for (int q = lane; q < tb / 16; q += 32)
+      for (int q = lane; q < tb / 16; q += kLanes)
         reinterpret_cast<uint4*>(stage)[q] = __ldg(reinterpret_cast<const uint4*>(src) + q);
     if (lane < area)
       old0 = atomicExch(&claim[base + (int64_t)(y + lane / sp) * fw + (x + lane % sp)], tag);
-    if (lane + 32 < area)
-      old1 = atomicExch(&claim[base + (int64_t)(y + (lane + 32) / sp) * fw + (x + (lane + 32) % sp)],
-                        tag);
-    for (int cell = lane + 64; cell < area; cell += 32)   // spans above 8
+    if (lane + kLanes < area)
+      old1 = atomicExch(
+          &claim[base + (int64_t)(y + (lane + kLanes) / sp) * fw + (x + (lane + kLanes) % sp)], tag);
+    for (int cell = lane + 2 * kLanes; cell < area; cell += kLanes)
       twice |= atomicExch(&claim[base + (int64_t)(y + cell / sp) * fw + (x + cell % sp)], tag) == tag;
     if (vec) {
-      __syncwarp();
+      __syncwarp(group);
       const int cpc = tb / 16;
-      for (int q = lane; q < area * cpc; q += 32) {
+      for (int q = lane; q < area * cpc; q += kLanes) {
         const int cell = q / cpc, j = q - cell * cpc;
         const int u = cell / sp, w = cell - u * sp;
         const int r0 = (2 * u) / sp, r1 = (2 * u + 1) / sp;
@@ -132,7 +134,7 @@ merge_nearest_warp_kernel(const T* __restrict__ mixed, int B, int N,
         reinterpret_cast<uint4*>(out + ocell * T4)[j] = chunk;
       }
     } else {
-      for (int task = lane; task < area * C; task += 32) {
+      for (int task = lane; task < area * C; task += kLanes) {
         const int cell = task / C, c = task - cell * C;
         const int u = cell / sp, w = cell - u * sp;
         const int r0 = (2 * u) / sp, r1 = (2 * u + 1) / sp;
@@ -625,10 +627,19 @@ merge_bilinear_tile_kernel(const T* __restrict__ mixed, int N, const int32_t* __
   }
 }
 
-// One pass up to here: us in one / two passes at 1945 tokens 3.2 / 4.0, 3890 5.6 /
-// 4.4, 7780 7.1 / 4.4, 124480 99 / 12.4 (64 x 64 cells per 1945 tokens, bf16; one
-// pass with 8 lanes per token and 4 CTAs per SM 3.2, 5.6, 4.9, 28.8).
-constexpr int kOnePassTokensPerSm = 16;
+// One pass, a warp per token, up to here: us in one / two passes at 1945 tokens
+// 3.2 / 4.0, 3040 4.0 / 4.5, 3890 5.4 / 4.5, 7780 7.1 / 4.4, 124480 99 / 12.4 (64 x 64
+// cells per 1945 tokens, bf16, 16 channels).
+constexpr int kOnePassTokensPerSm = 20;
+// Then 8 lanes per token while its output is small, where two passes are two
+// chains of latency: us with 8 lanes / two passes, 64 x 64 cells per 1945 tokens, 4
+// bf16 channels (67 bytes of output per token) 3890 tokens 3.2 / 4.6, 9725 3.7 / 4.8;
+// 8 channels (135) 3.6 / 4.6, 4.0 / 4.7; 16 channels (270) 4.0 / 4.5, 4.85 / 4.8.  With
+// spans up to 4 a few tokens have most of the cells: 4 channels (108) 3648 tokens 4.0
+// / 4.7, 9728 4.9 / 4.8; 8 channels (216) 5.3 / 4.8, 6.3 / 4.95.
+constexpr int kOnePassLanes = 8;
+constexpr int kOnePassSmallTokensPerSm = 64;
+constexpr int kOnePassSmallBytes = 144;
 constexpr int64_t kMaxWork = 0xfffffff0ll - 1024;   // 32-bit indices within an element
 constexpr int64_t kMaxGrid = 0x7fffffffll;
 
@@ -644,19 +655,26 @@ cudaError_t launch_t(const void* mixed, int B, int N, const int32_t* pos, const 
     cudaError_t e0 = cudaGetDevice(&dev);
     if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e0 != cudaSuccess) return e0;
-    cudaError_t e = prefer_max_shared<merge_nearest_warp_kernel<T>>();
+    cudaError_t e = prefer_max_shared<merge_nearest_warp_kernel<T, 32>>();
+    if (e == cudaSuccess) e = prefer_max_shared<merge_nearest_warp_kernel<T, kOnePassLanes>>();
     if (e == cudaSuccess) e = prefer_max_shared<merge_index_kernel>();
     if (e == cudaSuccess) e = prefer_max_shared<merge_nearest_gather_kernel<T, true>>();
     if (e == cudaSuccess) e = prefer_max_shared<merge_nearest_gather_kernel<T, false>>();
     if (e != cudaSuccess) return e;
     const bool whole = (C * 4 * (int)sizeof(T)) % 16 == 0;
     const int64_t work = (int64_t)fh * fw * (whole ? C * 4 * (int)sizeof(T) / 16 : C);
-    if (ntok <= (int64_t)std::max(1, sms) * kOnePassTokensPerSm || work > kMaxWork ||
-        B * ((work + 255) / 256) > kMaxGrid) {
-      // one warp per token, one pass (latency-bound sizes)
-      e = launch_pdl(merge_nearest_warp_kernel<T>, dim3((unsigned)((ntok + 7) / 8)),
-                     dim3(8 * 32), 0, s, static_cast<const T*>(mixed), B, N, pos, span, fh, fw,
-                     C, static_cast<T*>(out), hdr, words, status);
+    // one pass (latency-bound sizes)
+    const bool few = ntok <= (int64_t)std::max(1, sms) * kOnePassTokensPerSm || work > kMaxWork ||
+                     B * ((work + 255) / 256) > kMaxGrid;
+    const bool small = ntok <= (int64_t)std::max(1, sms) * kOnePassSmallTokensPerSm &&
+                       (int64_t)B * fh * fw * C * 4 * (int)sizeof(T) <= ntok * kOnePassSmallBytes;
+    if (few || small) {
+      const int toks = few ? 8 : 8 * 32 / kOnePassLanes;
+      e = launch_pdl(few ? merge_nearest_warp_kernel<T, 32>
+                         : merge_nearest_warp_kernel<T, kOnePassLanes>,
+                     dim3((unsigned)((ntok + toks - 1) / toks)), dim3(8 * 32), 0, s,
+                     static_cast<const T*>(mixed), B, N, pos, span, fh, fw, C,
+                     static_cast<T*>(out), hdr, words, status);
       if (e != cudaSuccess) return e;
       return cudaGetLastError();
     }

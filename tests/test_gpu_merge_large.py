@@ -84,6 +84,39 @@ def test_merge_two_pass_bit_exact(av, mode, dtype, C, B, fh, fw):
         assert _same(got, want)
 
 
+@pytest.mark.parametrize("spans", [[1, 2], [1, 3, 4], [1, 6, 12]])
+@pytest.mark.parametrize("dtype,C,B", [
+    ("bf16", 1, 20), ("bf16", 3, 20), ("bf16", 4, 20), ("f32", 1, 20),     # 8 lanes per token
+    ("bf16", 1, 90), ("bf16", 3, 90)])                                     # two passes
+def test_merge_nearest_routes(av, spans, dtype, C, B):
+    """Small tokens on both sides of the lines between one pass and two, with
+    spans whose cells are up to nine rounds of a token's eight lanes, a call with
+    a hole and one with a cell covered twice among good ones."""
+    import torch
+    import oracle
+    rng = np.random.default_rng(C + B + sum(spans))
+    fh, fw = 36, 24
+    ws = torch.zeros(av.avits_merge_final_workspace(NEAREST, B, fh, fw), dtype=torch.uint8, device="cuda")
+    # a span-1 block in every frame: at least 144 tokens an element
+    pos, span = _tiling(rng, B, fh, fw, 12, spans)
+    while pos.shape[1] < 144:
+        pos, span = _tiling(rng, B, fh, fw, 12, spans)
+    mixed = _latent(rng, B, pos.shape[1], C, dtype)
+    want, cover = oracle.merge_final(mixed, pos, span, fh, fw)
+    assert np.all(cover == 1)
+    for bad in (None, "hole", "twice", None):
+        p, s = pos.copy(), span.copy()
+        if bad == "hole":
+            s[B - 1, 3] = 0
+        elif bad == "twice":
+            one = np.flatnonzero(s[0] == 1)[:2]
+            p[0, one[1]] = p[0, one[0]]
+        got, st = _call(av, mixed, dtype, p, s, fh, fw, NEAREST, ws)
+        assert st == (0 if bad is None else 6)
+        if bad is None:
+            assert _same(got, want)
+
+
 @pytest.mark.parametrize("first", [NEAREST, BILINEAR])
 def test_merge_two_pass_reports_bad_tilings(av, first):
     import torch
