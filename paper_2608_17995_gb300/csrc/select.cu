@@ -574,11 +574,11 @@ select_upsample_kernel(const SelArgs g, const UpsampleArgs<T> u, int parts, int 
   if (staged) {
     const SharedRows<T> rows{rows_s, s_lo, T4};
     for (int i = lo + w; i < hi; i += kWarps)
-      upsample_token<T, kBilinear>(u, rows, b, i, offs_s[i], sel_s[i] != 0, lane);
+      upsample_token<T, kBilinear, false>(u, rows, b, i, offs_s[i], sel_s[i] != 0, lane);
   } else {
     const GlobalRows<T> rows{u.latent, M, T4};
     for (int i = lo + w; i < hi; i += kWarps)
-      upsample_token<T, kBilinear>(u, rows, b, i, offs_s[i], sel_s[i] != 0, lane);
+      upsample_token<T, kBilinear, false>(u, rows, b, i, offs_s[i], sel_s[i] != 0, lane);
   }
 }
 

@@ -15,7 +15,7 @@ namespace {
 
 constexpr int kWarpsPerCta = 8;
 
-template <typename T, bool kBilinear>
+template <typename T, bool kBilinear, bool kMapped>
 __global__ void __launch_bounds__(kWarpsPerCta * 32)
 upsample_kernel(const T* __restrict__ latent, int B, int M, int gh, int gw, int C,
                 const int32_t* __restrict__ pos_in, const int32_t* __restrict__ span_in,
@@ -33,7 +33,7 @@ upsample_kernel(const T* __restrict__ latent, int B, int M, int gh, int gw, int 
   const UpsampleArgs<T> u{latent, M, gh, gw, C, n_out, pos_in, span_in, out,
                           out_pos, out_span, out_src_tok, out_src_sub, map, status};
   const GlobalRows<T> rows{latent, M, C * 4};
-  upsample_token<T, kBilinear>(u, rows, b, i, tok_offset[in_tok], mask[in_tok] != 0, lane);
+  upsample_token<T, kBilinear, kMapped>(u, rows, b, i, tok_offset[in_tok], mask[in_tok] != 0, lane);
 }
 
 template <typename T>
@@ -45,8 +45,9 @@ cudaError_t launch_t(const void* latent, int B, int M, int gh, int gw, int C,
   const int64_t warps = (int64_t)B * M;
   const int grid = (int)((warps + kWarpsPerCta - 1) / kWarpsPerCta);
   const int n_out = M + 3 * k;
-  cudaError_t e = prefer_max_shared<upsample_kernel<T, true>>();
-  if (e == cudaSuccess) e = prefer_max_shared<upsample_kernel<T, false>>();
+  cudaError_t e = prefer_max_shared<upsample_kernel<T, false, false>>();
+  if (e == cudaSuccess) e = prefer_max_shared<upsample_kernel<T, true, false>>();
+  if (e == cudaSuccess) e = prefer_max_shared<upsample_kernel<T, true, true>>();
   if (e != cudaSuccess) return e;
   // bilinear with a mixed input: the input frame's cell map first
   int32_t* map = nullptr;
@@ -55,7 +56,9 @@ cudaError_t launch_t(const void* latent, int B, int M, int gh, int gw, int C,
     e = launch_cell_map(B, M, pos_in, span_in, gh, gw, map, status, s);
     if (e != cudaSuccess) return e;
   }
-  auto kern = (mode == AVITS_UP_BILINEAR) ? upsample_kernel<T, true> : upsample_kernel<T, false>;
+  auto kern = map                         ? upsample_kernel<T, true, true>
+              : mode == AVITS_UP_BILINEAR ? upsample_kernel<T, true, false>
+                                          : upsample_kernel<T, false, false>;
   e = launch_pdl(kern, dim3(grid), dim3(kWarpsPerCta * 32), 0, s,
                  static_cast<const T*>(latent), B, M, gh, gw, C, pos_in, span_in, mask,
                  tok_offset, n_out, static_cast<T*>(out), out_pos, out_span, out_src_tok,

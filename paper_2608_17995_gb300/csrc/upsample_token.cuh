@@ -123,8 +123,9 @@ __device__ __forceinline__ uint4 bilinear_child(const Src& rows, int b_elem, int
 
 // Token i of element b, selected or not, starting at output o; one warp.
 // Src::row(b, tok) gives the token's source values (tok's bilinear
-// neighbours included).
-template <typename T, bool kBilinear, typename Src>
+// neighbours included).  kMapped: bilinear from the frame's pyramid (u.map), an
+// instance of its own (in one with the dense grid's 16-byte pieces it lost 3 %).
+template <typename T, bool kBilinear, bool kMapped, typename Src>
 __device__ __forceinline__ void upsample_token(const UpsampleArgs<T>& u, const Src& rows, int b,
                                                int i, int o, bool sel, int lane) {
   using PV = typename Pix4<T>::V;
@@ -151,8 +152,9 @@ __device__ __forceinline__ void upsample_token(const UpsampleArgs<T>& u, const S
   const T* src = rows.row(b, i);
   const int64_t out_tok0 = (int64_t)b * u.n_out + o;
   const int tb = T4 * (int)sizeof(T);
-  const bool pieces = Chunk<T>::kCh == 1 || 4 * C > 32;   // of bilinear children
-  if ((tb & 15) == 0 && (!kBilinear || !sel || (pieces && !u.map))) {
+  // bilinear children in pieces
+  const bool pieces = !kMapped && (Chunk<T>::kCh == 1 || 4 * C > 32);
+  if ((tb & 15) == 0 && (!kBilinear || !sel || pieces)) {
     // 16-byte chunks: a deferred token is copied; nearest gives each child
     // (a, b) of a selected one the chunk whose channel pixels all equal the
     // parent's pixel (a, b), bilinear on a dense grid resizes around it; one
@@ -166,7 +168,7 @@ __device__ __forceinline__ void upsample_token(const UpsampleArgs<T>& u, const S
         const int child = q / cpc, j = q - child * cpc;
         const int a = child >> 1, bb = child & 1;
         uint4 w;
-        if constexpr (kBilinear)
+        if constexpr (kBilinear && !kMapped)
           w = bilinear_child<T>(rows, b, gh, gw, y, x, a, bb, j);
         else
           w = gather_chunk<T>(src, j, a, a, bb, bb);
@@ -188,7 +190,7 @@ __device__ __forceinline__ void upsample_token(const UpsampleArgs<T>& u, const S
       const int child = task / C, c = task - child * C;
       const int a = child >> 1, bb = child & 1;
       PV v;
-      if (kBilinear && u.map) {
+      if constexpr (kMapped) {
         float r[4] = {0.f, 0.f, 0.f, 0.f};
         if (frame_ok) {
           const T* tokb = u.latent + (int64_t)b * M * T4;
@@ -199,7 +201,7 @@ __device__ __forceinline__ void upsample_token(const UpsampleArgs<T>& u, const S
             r[q] = frame_resize2x(lv, tokb, T4, mapb, gh, gw, c, R0 + (q >> 1), Q0 + (q & 1));
         }
         v = Pix4<T>::make(r[0], r[1], r[2], r[3]);
-      } else if (!kBilinear) {
+      } else if constexpr (!kBilinear) {
         const float p = load_elem(src, c * 4 + a * 2 + bb);
         v = Pix4<T>::make(p, p, p, p);
       } else {
