@@ -8,7 +8,7 @@
 // 32 different rows (no bytes read twice by a warp) and a query row's are one
 // broadcast.  Every dot product keeps four partial sums (columns c mod 4).  Q
 // and K come in chunks of 32 columns through a 3-stage ring (cp.async for
-// fp32).  After a key tile each lane folds its logits into a running (max, sum
+// fp32, 16-byte loads through registers for bf16).  After a key tile each lane folds its logits into a running (max, sum
 // over all keys, sum over text keys) per query in the log2 domain; the lanes
 // are merged by shuffles only when the head's keys end.
 //
@@ -27,7 +27,9 @@
 // latency with 8 warps per SM.  24 heads x 1024 x 1536 x 128 fp32: 3950 -> 310
 // us (31 of 74 TFLOP/s; before, one warp per query read each key row for four
 // FMAs per 16-byte load, and heads ran one after the other); 2 heads x 256 x
-// 288 x 64: 17 -> 6.7 us.  Packed f32x2 FMAs, pairs of columns or of keys,
+// 288 x 64: 17 -> 6.7 us.  bf16: 24 heads x 1024 x 1536 x 96 2125 -> 317 us (457 with
+// elements loaded one by one), x 40 979 -> 180 (259), 8 x 16 heads x 256 x 333 x 256
+// 1378 -> 258 (380), 1 head x 64 x 100 x 256 10.5 -> 10.3 (21.9).  Packed f32x2 FMAs, pairs of columns or of keys,
 // were no faster (411 us either way with 8 x 4 lanes to a warp's tile), nor
 // were 64 rows per CTA (615-640 us, one CTA per SM).
 #include "avits_common.cuh"
@@ -98,10 +100,15 @@ struct SimtParams {
   int tiles, n_kt, items, per, cs;   // query tiles; items and items per CTA of a cluster
 };
 
+// How a stage's rows come to shared memory.  Elements: one by one.  Async: fp32 in
+// 16-byte asynchronous copies.  Vectors: bf16 in 16-byte loads into registers,
+// converted and stored once the products of the stage in hand have been issued.
+// The last two need d, the strides and the bases to be multiples of 16 bytes
+// (checked on the host).
+enum Load { kLoadElements, kLoadAsync, kLoadVectors };
+
 // kRows rows (row r0 + r of `base`, valid below `rows`) of columns c0 ..
 // c0 + 31 (below d) into ks as fp32, zero where there is no element.
-// kAsync: fp32 in 16-byte asynchronous copies (d, the strides and the base
-// are multiples of them, checked on the host); otherwise element by element.
 template <typename T, int kRows, int kThreads, bool kAsync>
 __device__ __forceinline__ void load_rows(const T* base, int64_t sn, int r0, int rows, int c0,
                                           int d, float* ks) {
@@ -137,13 +144,45 @@ __device__ __forceinline__ void load_rows(const T* base, int64_t sn, int r0, int
   }
 }
 
+// A stage of bf16 (kQ query rows, then kTN key rows) in registers on its way to
+// shared memory: 8 columns per vector, four vectors per row.
+template <int kQ, int kThreads>
+struct StageVectors {
+  static constexpr int kN = ((kQ + kTN) * 4 + kThreads - 1) / kThreads;
+  uint4 w[kN];
+  __device__ __forceinline__ void load(const __nv_bfloat16* q, int64_t q_sn, int q0, int q_rows,
+                                       const __nv_bfloat16* k, int64_t k_sn, int k0, int k_rows,
+                                       int c0, int d) {
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+      const int v = threadIdx.x + u * kThreads, c = c0 + (v & 3) * 8;
+      const int r = v >> 2;
+      const bool of_q = r < kQ;
+      const int row = of_q ? q0 + r : k0 + (r - kQ);
+      w[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (r < kQ + kTN && row < (of_q ? q_rows : k_rows) && c < d)
+        w[u] = *reinterpret_cast<const uint4*>((of_q ? q + (int64_t)row * q_sn : k + (int64_t)row * k_sn) + c);
+    }
+  }
+  __device__ __forceinline__ void store(float* st) const {
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+      const int v = threadIdx.x + u * kThreads, r = v >> 2;
+      if (r >= kQ + kTN) continue;
+      float4* dst = reinterpret_cast<float4*>(st + r * kLd + (v & 3) * 8);
+      dst[0] = make_float4(bf16_lo(w[u].x), bf16_hi(w[u].x), bf16_lo(w[u].y), bf16_hi(w[u].y));
+      dst[1] = make_float4(bf16_lo(w[u].z), bf16_hi(w[u].z), bf16_lo(w[u].w), bf16_hi(w[u].w));
+    }
+  }
+};
+
 template <int TM>
 constexpr size_t simt_smem() {
   return (size_t)kStages * (TM + kTN) * kLd * sizeof(float);
 }
 
-template <typename T, int TM, int RM, bool kAsync>
-__global__ void __launch_bounds__(32 * (TM / RM), TM / RM > 4 ? 1 : 2)
+template <typename T, int TM, int RM, Load kLoad>
+__global__ void __launch_bounds__(32 * (TM / RM), 2)
 spatial_simt_kernel(const SimtParams p) {
   constexpr int kThreads = 32 * (TM / RM);
   constexpr int kStageFloats = (TM + kTN) * kLd;
@@ -168,16 +207,26 @@ spatial_simt_kernel(const SimtParams p) {
   const int nch = (p.d + kDK - 1) / kDK;
   const float ln2 = 0.69314718055994530942f;
 
-  // the load side runs two stages ahead
+  // the load side runs two stages ahead; vectors: the registers of a stage are
+  // loaded by issue() and stored by deliver()
+  StageVectors<TM, kThreads> held;
+  float* held_for = nullptr;
   int l_it = it_begin, l_ch = 0, l_stage = 0;
   int l_h = it_begin / p.n_kt, l_kt = it_begin - l_h * p.n_kt;
   auto issue = [&]() {
     if (l_it < it_end) {
       float* st = stages + l_stage * kStageFloats;
-      load_rows<T, TM, kThreads, kAsync>(qb + (int64_t)l_h * p.q_sh, p.q_sn, row0, p.M,
-                                         l_ch * kDK, p.d, st);
-      load_rows<T, kTN, kThreads, kAsync>(kb + (int64_t)l_h * p.k_sh, p.k_sn, l_kt * kTN, p.Nk,
-                                          l_ch * kDK, p.d, st + TM * kLd);
+      if constexpr (kLoad == kLoadVectors) {
+        held.load(qb + (int64_t)l_h * p.q_sh, p.q_sn, row0, p.M, kb + (int64_t)l_h * p.k_sh, p.k_sn,
+                  l_kt * kTN, p.Nk, l_ch * kDK, p.d);
+        held_for = st;
+      } else {
+        load_rows<T, TM, kThreads, kLoad == kLoadAsync>(qb + (int64_t)l_h * p.q_sh, p.q_sn, row0, p.M,
+                                                        l_ch * kDK, p.d, st);
+        load_rows<T, kTN, kThreads, kLoad == kLoadAsync>(kb + (int64_t)l_h * p.k_sh, p.k_sn,
+                                                         l_kt * kTN, p.Nk, l_ch * kDK, p.d,
+                                                         st + TM * kLd);
+      }
       if (++l_ch == nch) {
         l_ch = 0;
         ++l_it;
@@ -187,8 +236,16 @@ spatial_simt_kernel(const SimtParams p) {
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  auto deliver = [&]() {
+    if constexpr (kLoad == kLoadVectors) {
+      if (held_for) held.store(held_for);
+      held_for = nullptr;
+    }
+  };
   issue();
+  deliver();
   issue();
+  deliver();
 
   RowStat st[RM];
 #pragma unroll
@@ -242,6 +299,7 @@ spatial_simt_kernel(const SimtParams p) {
 #pragma unroll 1
         for (int c = 0; c < left; c += 4) step(c);
       }
+      deliver();
     }
     // fold the tile's logits into the row statistics
     const int key0 = kt * kTN + lane;
@@ -393,7 +451,7 @@ Plan make_plan(int B, int H, int M, int Nk, int num_sms) {
   return pl;
 }
 
-template <typename T, int TM, int RM, bool kAsync>
+template <typename T, int TM, int RM, Load kLoad>
 cudaError_t launch_one(const SimtParams& p, cudaStream_t s) {
   // the shared-memory opt-in, once per device
   static int done[64] = {};
@@ -401,9 +459,9 @@ cudaError_t launch_one(const SimtParams& p, cudaStream_t s) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (!(dev >= 0 && dev < 64 && __atomic_load_n(&done[dev], __ATOMIC_ACQUIRE))) {
-    e = cudaFuncSetAttribute(spatial_simt_kernel<T, TM, RM, kAsync>,
+    e = cudaFuncSetAttribute(spatial_simt_kernel<T, TM, RM, kLoad>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)simt_smem<TM>());
-    if (e == cudaSuccess) e = prefer_max_shared<spatial_simt_kernel<T, TM, RM, kAsync>>();
+    if (e == cudaSuccess) e = prefer_max_shared<spatial_simt_kernel<T, TM, RM, kLoad>>();
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) __atomic_store_n(&done[dev], 1, __ATOMIC_RELEASE);
   }
@@ -421,15 +479,15 @@ cudaError_t launch_one(const SimtParams& p, cudaStream_t s) {
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, spatial_simt_kernel<T, TM, RM, kAsync>, p);
+  e = cudaLaunchKernelEx(&cfg, spatial_simt_kernel<T, TM, RM, kLoad>, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
-template <typename T, bool kAsync>
+template <typename T, Load kLoad>
 cudaError_t launch_typed(const SimtParams& p, int tm, cudaStream_t s) {
-  if (tm == 32) return launch_one<T, 32, 8, kAsync>(p, s);
-  return launch_one<T, 16, 4, kAsync>(p, s);
+  if (tm == 32) return launch_one<T, 32, 8, kLoad>(p, s);
+  return launch_one<T, 16, 4, kLoad>(p, s);
 }
 
 }  // namespace
@@ -451,13 +509,17 @@ cudaError_t launch_spatial_simt(const SpatialArgs& a, int num_sms, cudaStream_t 
   p.per = pl.per;
   p.cs = pl.cs;
   if ((int64_t)a.B * p.tiles * p.cs > 0x7fffffff) return cudaErrorInvalidValue;
-  if (a.dt == AVITS_BF16) return launch_typed<__nv_bfloat16, false>(p, pl.tm, s);
-  // 16-byte copies: d, the strides and both bases multiples of 4 floats
+  // 16-byte loads: d, the strides and both bases multiples of 16 bytes
+  const int64_t n = a.dt == AVITS_BF16 ? 8 : 4;   // elements
   const bool vec = ((reinterpret_cast<uintptr_t>(a.q) | reinterpret_cast<uintptr_t>(a.k)) & 15u) == 0 &&
-                   a.d % 4 == 0 && a.q_sn % 4 == 0 && a.k_sn % 4 == 0 &&
-                   (a.H == 1 || (a.q_sh % 4 == 0 && a.k_sh % 4 == 0)) &&
-                   (a.B == 1 || (a.q_sb % 4 == 0 && a.k_sb % 4 == 0));
-  return vec ? launch_typed<float, true>(p, pl.tm, s) : launch_typed<float, false>(p, pl.tm, s);
+                   a.d % n == 0 && a.q_sn % n == 0 && a.k_sn % n == 0 &&
+                   (a.H == 1 || (a.q_sh % n == 0 && a.k_sh % n == 0)) &&
+                   (a.B == 1 || (a.q_sb % n == 0 && a.k_sb % n == 0));
+  if (a.dt == AVITS_BF16)
+    return vec ? launch_typed<__nv_bfloat16, kLoadVectors>(p, pl.tm, s)
+               : launch_typed<__nv_bfloat16, kLoadElements>(p, pl.tm, s);
+  return vec ? launch_typed<float, kLoadAsync>(p, pl.tm, s)
+             : launch_typed<float, kLoadElements>(p, pl.tm, s);
 }
 
 }  // namespace avits

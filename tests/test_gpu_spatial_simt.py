@@ -78,6 +78,39 @@ def test_simt_edges(av, dtype, B, H, M, L, R, d, mask):
         assert torch.equal(A, A2)   # the same sums in the same order
 
 
+@pytest.mark.parametrize("B,H,M,L,R,d", [
+    (1, 1, 1, 1, 0, 8),             # one row, one vector
+    (1, 1, 64, 36, 0, 256),         # one key tile of 100
+    (2, 3, 17, 111, 0, 40),         # a last chunk of one vector
+    (1, 2, 300, 77, 640, 96),
+    (3, 24, 700, 33, 0, 32),        # 32-row tiles, the last of 28 rows
+    (16, 1, 70, 26, 0, 264 - 16),   # eight chunks, the last of three vectors
+])
+def test_simt_bf16_vectors(av, B, H, M, L, R, d):
+    """bf16 in 16-byte loads: the oracle's values, and the bits of the
+    element-wise loads that a misaligned view takes."""
+    import torch
+    import oracle
+    from paper_2608_17995_gb300.pipeline import to_numpy
+    g = torch.Generator(device="cuda").manual_seed(M + d)
+    N, scale = L + M + R, 1.0 / math.sqrt(d)
+    q = (math.sqrt(2.0) * torch.randn(B, H, M, d, generator=g, device="cuda")).bfloat16()
+    k = (math.sqrt(2.0) * torch.randn(B, H, N, d, generator=g, device="cuda")).bfloat16()
+    A, A2 = torch.zeros(B, M, device="cuda"), torch.zeros(B, M, device="cuda")
+    av.avits_score_spatial(q, k, L, scale, A)
+    buf = torch.zeros(B, N, H, d + 1, device="cuda", dtype=torch.bfloat16)[..., 1:]
+    buf.copy_(k.transpose(1, 2))
+    av.avits_score_spatial(q, buf.transpose(1, 2), L, scale, A2)
+    assert av.avits_device_status() == 0
+    assert torch.equal(A, A2)
+    # token-major rows of whole vectors keep the 16-byte loads
+    av.avits_score_spatial(q, k.transpose(1, 2).contiguous().transpose(1, 2), L, scale, A2)
+    assert av.avits_device_status() == 0
+    assert torch.equal(A, A2)
+    want = oracle.score_spatial(to_numpy(q), to_numpy(k), L, scale)[0]
+    np.testing.assert_allclose(to_numpy(A), want, rtol=TOL, atol=1e-7)
+
+
 def test_simt_no_finite_key(av):
     """NaN and infinite logits give NaN for their rows alone."""
     import torch
