@@ -20,6 +20,12 @@ constexpr int kMapLevelShift = 28;
 constexpr int32_t kMapTokMask = (1 << kMapLevelShift) - 1;
 constexpr int kMaxMapLevel = 2;   // spans 1, 2 and 4
 
+// Whether a token of s x s cells at (y, x) lies in a frame of fh x fw cells, for
+// any values (no sum that could overflow).
+__device__ __forceinline__ bool in_frame(int y, int x, int s, int fh, int fw) {
+  return s > 0 && y >= 0 && x >= 0 && s <= fh - y && s <= fw - x;
+}
+
 __device__ __forceinline__ int32_t map_entry(int tok, int lvl) {
   return tok | (lvl << kMapLevelShift);
 }

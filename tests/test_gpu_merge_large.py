@@ -117,6 +117,31 @@ def test_merge_nearest_routes(av, spans, dtype, C, B):
             assert _same(got, want)
 
 
+@pytest.mark.parametrize("mode", [NEAREST, BILINEAR])
+@pytest.mark.parametrize("dtype,C,B", [("bf16", 16, 1), ("bf16", 4, 20), ("bf16", 16, 20), ("bf16", 3, 20),
+                                       ("bf16", 3, 80)])
+def test_positions_and_spans_beyond_the_integers(av, mode, dtype, C, B):
+    """A token whose last row or column does not fit an int is outside the frame
+    like any other: reported, its cells are holes, and the next call is right."""
+    import torch
+    import oracle
+    rng = np.random.default_rng(C + B)
+    fh, fw, top = 24, 24, 2 ** 31 - 1
+    pos, span = _tiling(rng, B, fh, fw, 4, [1, 2])
+    mixed = _latent(rng, B, pos.shape[1], C, dtype)
+    want, _ = oracle.merge_final(mixed, pos, span, fh, fw, mode="nearest" if mode == NEAREST else "bilinear")
+    ws = torch.zeros(av.avits_merge_final_workspace(mode, B, fh, fw), dtype=torch.uint8, device="cuda")
+    for at, s in (([top, 0], None), ([0, top], None), ([top - 1, top - 1], None), ([1, 0], top),
+                  ([top, top], top), ([-top - 1, 3], top)):
+        p, sp = pos.copy(), span.copy()
+        p[B - 1, 5] = at
+        if s is not None:
+            sp[B - 1, 5] = s
+        assert _call(av, mixed, dtype, p, sp, fh, fw, mode, ws)[1] == 6
+    got, st = _call(av, mixed, dtype, pos, span, fh, fw, mode, ws)
+    assert st == 0 and _same(got, want)
+
+
 @pytest.mark.parametrize("first", [NEAREST, BILINEAR])
 def test_merge_two_pass_reports_bad_tilings(av, first):
     import torch
