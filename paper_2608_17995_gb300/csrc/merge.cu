@@ -629,8 +629,12 @@ merge_bilinear_tile_kernel(const T* __restrict__ mixed, int N, const int32_t* __
 
 // One pass, a warp per token, up to here: us in one / two passes at 1945 tokens
 // 3.2 / 4.0, 3040 4.0 / 4.5, 3890 5.4 / 4.5, 7780 7.1 / 4.4, 124480 99 / 12.4 (64 x 64
-// cells per 1945 tokens, bf16, 16 channels).
-constexpr int kOnePassTokensPerSm = 20;
+// cells per 1945 tokens, bf16, 16 channels: 270 bytes of output per token).  The
+// second line holds for tokens of up to so many bytes of output (12 fp32 channels,
+// 404 bytes, 3040 tokens: 5.1 / 4.4).
+constexpr int kOnePassTokensPerSm = 16;
+constexpr int kOnePassMoreTokensPerSm = 20;
+constexpr int kOnePassMoreBytes = 288;
 // Then 8 lanes per token while its output is small, where two passes are two
 // chains of latency: us with 8 lanes / two passes, 64 x 64 cells per 1945 tokens, 4
 // bf16 channels (67 bytes of output per token) 3890 tokens 3.2 / 4.6, 9725 3.7 / 4.8;
@@ -664,10 +668,12 @@ cudaError_t launch_t(const void* mixed, int B, int N, const int32_t* pos, const 
     const bool whole = (C * 4 * (int)sizeof(T)) % 16 == 0;
     const int64_t work = (int64_t)fh * fw * (whole ? C * 4 * (int)sizeof(T) / 16 : C);
     // one pass (latency-bound sizes)
-    const bool few = ntok <= (int64_t)std::max(1, sms) * kOnePassTokensPerSm || work > kMaxWork ||
-                     B * ((work + 255) / 256) > kMaxGrid;
-    const bool small = ntok <= (int64_t)std::max(1, sms) * kOnePassSmallTokensPerSm &&
-                       (int64_t)B * fh * fw * C * 4 * (int)sizeof(T) <= ntok * kOnePassSmallBytes;
+    const auto up_to = [&](int per_sm) { return ntok <= (int64_t)std::max(1, sms) * per_sm; };
+    const int64_t out_bytes = (int64_t)B * fh * fw * C * 4 * (int)sizeof(T);
+    const bool few = up_to(kOnePassTokensPerSm) ||
+                     (up_to(kOnePassMoreTokensPerSm) && out_bytes <= ntok * kOnePassMoreBytes) ||
+                     work > kMaxWork || B * ((work + 255) / 256) > kMaxGrid;
+    const bool small = up_to(kOnePassSmallTokensPerSm) && out_bytes <= ntok * kOnePassSmallBytes;
     if (few || small) {
       const int toks = few ? 8 : 8 * 32 / kOnePassLanes;
       e = launch_pdl(few ? merge_nearest_warp_kernel<T, 32>
