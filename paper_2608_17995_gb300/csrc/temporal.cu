@@ -1,13 +1,14 @@
 // temporal.cu — temporal importance (Sec. 3.3.2).
 //
 // avits_score_temporal: V = ||h_t - h_prev|| / (||h_prev|| + eps) per token.
-// HBM-bound.  Main path: each CTA stages up to 8 token rows of both
+// HBM-bound.  Main path: each CTA stages a chunk of token rows of both
 // snapshots in shared memory with bulk copies (cp.async.bulk, one per row,
 // completing on one mbarrier), so a whole chunk is in flight with a single
 // issuing thread; then one warp per token reduces its two rows from shared
-// memory (fp32 sums, shuffle reduction).  Chunks are small (2 tokens) and
-// many CTAs fit on an SM, so all of the input is in flight at once and the
-// kernel can share SMs with the spatial kernel.  Rows that are not 16-byte
+// memory (fp32 sums, shuffle reduction).  Chunks are small (2 tokens; beside the
+// spatial kernel up to 24 KB of narrow rows) and many CTAs fit on an SM, so all of
+// the input is in flight at once and the kernel can share SMs with the spatial
+// kernel.  Rows that are not 16-byte
 // multiples use a register path.  Algorithmic bytes: 2 * B*N*D*elt + 4*B*N.
 //
 // avits_score_temporal_var: Eq. 6-7, unbiased variance over N_T snapshots

@@ -79,7 +79,9 @@ class TransitionBuffers:
         self.q, self.k, self.h_t, self.h_prev, self.latent = q, k, h_t, h_prev, latent
         self.pos_in, self.span_in = pos_in, span_in
 
-    # the five steps, each one launch (the bilinear merge adds a memset + map)
+    # the five steps, each one launch, but for the merge of larger batches (two)
+    # and the bilinear one (two or three), and a mixed bilinear upsample (its cell
+    # map: two more)
     def spatial(self, stream=None):
         avits_score_spatial(self.q, self.k, self.tr.L, self.tr.softmax_scale, self.A,
                             workspace=self.ws, stream=stream)
