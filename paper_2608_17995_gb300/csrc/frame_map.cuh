@@ -2,7 +2,8 @@
 // pyramid that multi-level bilinear resampling reads (Sec. 3.2, Stages 2-3).
 //
 // A frame of fh x fw cells is tiled by tokens of span s in {1, 2, 4}, each at
-// a multiple of s; token pixel (a, b) stands for the s x s full pixels
+// a multiple of s (a token is looked for outside the frame by y > fh - s, which
+// unlike y + s > fh cannot overflow); token pixel (a, b) stands for the s x s full pixels
 // (2y + a*s .., 2x + b*s ..).  The map holds, per cell, the covering token's
 // index within its element and log2(s).  Level l of the pyramid: a level-l
 // pixel inside one token pixel (span >= 2^l) is that pixel; any other is
@@ -19,12 +20,6 @@ namespace avits {
 constexpr int kMapLevelShift = 28;
 constexpr int32_t kMapTokMask = (1 << kMapLevelShift) - 1;
 constexpr int kMaxMapLevel = 2;   // spans 1, 2 and 4
-
-// Whether a token of s x s cells at (y, x) lies in a frame of fh x fw cells, for
-// any values (no sum that could overflow).
-__device__ __forceinline__ bool in_frame(int y, int x, int s, int fh, int fw) {
-  return s > 0 && y >= 0 && x >= 0 && s <= fh - y && s <= fw - x;
-}
 
 __device__ __forceinline__ int32_t map_entry(int tok, int lvl) {
   return tok | (lvl << kMapLevelShift);

@@ -89,7 +89,7 @@ merge_nearest_warp_kernel(const T* __restrict__ mixed, int B, int N,
     y = pos[t * 2];
     x = pos[t * 2 + 1];
     sp = span[t];
-    valid = in_frame(y, x, sp, fh, fw);
+    valid = !(sp <= 0 || y < 0 || x < 0 || y > fh - sp || x > fw - sp);
     if (!valid && lane == 0) raise_status(status, AVITS_ERR_COVERAGE);
   }
   __syncthreads();   // cta_cells is initialised
@@ -180,7 +180,7 @@ merge_index_kernel(int B, int N, const int32_t* __restrict__ pos, const int32_t*
     x = pos[t * 2 + 1];
     s = span[t];
     base = (int64_t)b * fh * fw;
-    if (!in_frame(y, x, s, fh, fw)) {
+    if (s <= 0 || y < 0 || x < 0 || y > fh - s || x > fw - s) {
       raise_status(status, AVITS_ERR_COVERAGE);
       s = 0;
     }
@@ -257,7 +257,7 @@ merge_nearest_gather_kernel(const T* __restrict__ mixed, int N, const int32_t* _
     const int Y = (int)(cell[k] / (unsigned)fw), X = (int)(cell[k] % (unsigned)fw);
     const int u = Y - y[k], w = X - x[k], sp = s[k];
     if (t[k] < 0 || u < 0 || w < 0 || u >= sp || w >= sp || y[k] < 0 || x[k] < 0 ||
-        sp > fh - y[k] || sp > fw - x[k]) {
+        y[k] > fh - sp || x[k] > fw - sp) {
       raise_status(status, AVITS_ERR_COVERAGE);
       continue;
     }
@@ -294,7 +294,7 @@ __global__ void merge_map_kernel(int B, int N, const int32_t* __restrict__ pos,
   const int b = (int)(t / N), ti = (int)(t % N);
   const int y = pos[t * 2], x = pos[t * 2 + 1], s = span[t];
   const int lvl = (s == 1) ? 0 : (s == 2) ? 1 : (s == 4) ? 2 : -1;
-  if (lvl < 0 || !in_frame(y, x, s, fh, fw) || ((y | x) & (s - 1))) {
+  if (lvl < 0 || y < 0 || x < 0 || y > fh - s || x > fw - s || ((y | x) & (s - 1))) {
     raise_status(status, AVITS_ERR_COVERAGE);
     return;
   }
@@ -340,7 +340,7 @@ merge_scatter_kernel(int B, int N, const int32_t* __restrict__ pos,
     const int b = (int)(t / N), ti = (int)(t - (int64_t)b * N);
     const int y = pos[t * 2], x = pos[t * 2 + 1], s = span[t];
     const int lvl = (s == 1) ? 0 : (s == 2) ? 1 : (s == 4) ? 2 : -1;
-    if (lvl < 0 || !in_frame(y, x, s, fh, fw) || ((y | x) & (s - 1))) {
+    if (lvl < 0 || y < 0 || x < 0 || y > fh - s || x > fw - s || ((y | x) & (s - 1))) {
       raise_status(status, AVITS_ERR_COVERAGE);
     } else {
       const int32_t entry = map_entry(ti, lvl);
@@ -373,7 +373,7 @@ struct CellWord {
   // there).  Only a word that passed here may be followed to a token.
   __device__ int32_t live(int N, int fh, int fw, int Y, int X) const {
     const bool ok = e >= 0 && map_lvl(e) <= kMaxMapLevel && map_tok(e) < N && s == 1 << map_lvl(e) &&
-                    (Y & ~(s - 1)) == y && (X & ~(s - 1)) == x && in_frame(y, x, s, fh, fw);
+                    (Y & ~(s - 1)) == y && (X & ~(s - 1)) == x && y <= fh - s && x <= fw - s;
     return ok ? e : -1;
   }
 };

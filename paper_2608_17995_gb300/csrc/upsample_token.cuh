@@ -184,7 +184,8 @@ __device__ __forceinline__ void upsample_token(const UpsampleArgs<T>& u, const S
     // frame's pyramid; an invalid position or span (reported by the map
     // kernel) gives zeros
     const int lv = (s == 1) ? 0 : (s == 2) ? 1 : (s == 4) ? 2 : -1;
-    const bool frame_ok = lv >= 0 && in_frame(y, x, s, gh, gw) && ((y | x) & (s - 1)) == 0;
+    const bool frame_ok = lv >= 0 && y >= 0 && x >= 0 && y <= gh - s && x <= gw - s &&
+                          ((y | x) & (s - 1)) == 0;
     for (int task = lane; task < 4 * C; task += 32) {
       const int child = task / C, c = task - child * C;
       const int a = child >> 1, bb = child & 1;
